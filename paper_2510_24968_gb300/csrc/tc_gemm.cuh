@@ -1,17 +1,30 @@
-// BF16 x BF16 -> FP32 GEMM on the fifth-generation tensor cores for the
-// learned-guess network: C[M x N] = op(A)[M x K] op(B)[K x N] (+ bias[N]).
+// BF16 x BF16 -> FP32 GEMMs on the fifth-generation tensor cores for the
+// learned-guess network, with its element-wise steps as epilogues.
 //
-// One CTA of four warps per 128 x 128 tile of C.  The K dimension is walked in
-// chunks of 64: all threads stage the chunk of A (128 rows) and of op(B)^T
-// (128 columns of C) into shared memory as BF16, in the canonical no-swizzle
-// K-major layout (core matrices of 8 rows x 16 bytes, 128 contiguous bytes
-// each); one thread issues four tcgen05.mma (M 128, N 128, K 16 each) that
-// accumulate in tensor memory (128 lanes x 128 FP32 columns) and commits them
-// to an mbarrier, which every thread waits on (bounded) before the next chunk
-// overwrites the operands.  The epilogue reads the accumulator back with
-// tcgen05.ld (warp w: lanes, i.e. rows, 32w .. 32w + 31), adds the bias and
-// stores FP32.  A wait that runs out sets *err and the CTA frees its tensor
-// memory and returns.
+// One CTA of four warps per 128 x 128 tile of the product.  The K dimension is
+// walked in chunks of 64, each staged into shared memory in the canonical
+// no-swizzle K-major layout (core matrices of 8 rows x 16 bytes, 128 contiguous
+// bytes each); one thread issues four tcgen05.mma (M 128, N 128, K 16 each)
+// that accumulate in tensor memory (128 lanes x 128 FP32 columns) and commits
+// them to the chunk's mbarrier.  Then the accumulator goes through shared
+// memory (tcgen05.ld gives a thread one row; the epilogue wants a column) and
+// thread t runs the epilogue on column t of the tile, row by row: global
+// accesses coalesce and a column sum is one register.  A wait that runs out
+// sets *err and the CTA frees its tensor memory and returns.
+//
+//  * tc_layer_kernel: forward layers and the data gradients.  Both operands lie
+//    in memory K-contiguous, BF16, zero-padded to whole chunks (activations as
+//    the previous epilogue left them, weights packed once per update), so a
+//    chunk is 16 cp.async of 16 bytes per thread, kTcStages chunks in flight:
+//    at K <= 256 every load is issued before the first MMA.
+//  * tc_wgrad_kernel: weight gradients, K = the batch.  256 x 256 outputs are
+//    only four tiles, so the batch is split over CTAs (partial products in a
+//    workspace, summed in order by the caller: repeated calls give the same
+//    bits), all layers in one launch; operands are batch-major and transposed
+//    while they are staged (eight coalesced row loads per 16-byte unit).
+// What bounds them is latency, not the tensor pipe (1.6 GFLOP in all): at batch
+// 4096, width 256, a gradient took 4.4 ms when every GEMM staged 2-byte elements
+// through FP32 loads and the weight gradients ran on 2-4 CTAs (1.1 ms each);
 #pragma once
 #include <cuda_bf16.h>
 
@@ -22,12 +35,19 @@ namespace fsim {
 constexpr int kTcM = 128, kTcN = 128, kTcK = 64;
 constexpr int kTcThreads = 128;
 constexpr uint32_t kTcStage = (uint32_t)kTcM * kTcK * 2;  // bytes of one operand chunk
-// dynamic shared memory per CTA: the two chunks (16 KB each), alignment slack
-// and the barrier, rounded up so that at most three CTAs share an SM and their
-// tensor-memory allocations (3 x 128 columns) fit the SM's 512 columns
-constexpr int kTcSmemBytes = 60 * 1024;
-static_assert(2 * kTcStage + 1024 + 64 <= (uint32_t)kTcSmemBytes, "tile does not fit");
-static_assert(4 * kTcSmemBytes > 227 * 1024, "four CTAs per SM would oversubscribe tensor memory");
+constexpr int kTcStages = 4;                      // chunks in flight, layers
+constexpr int kTcWStages = 2;                     // chunks in flight, weight gradients
+constexpr int kTcTileLd = kTcN + 1;               // accumulator tile in shared memory, padded against conflicts
+constexpr uint32_t kTcTile = (uint32_t)kTcM * kTcTileLd * 4;
+// dynamic shared memory per CTA: the larger of the operand ring and the
+// accumulator tile (which reuses it), alignment slack and the barriers; at most
+// three CTAs then share an SM and their tensor-memory allocations (3 x 128
+// columns) fit the SM's 512 columns
+__host__ __device__ constexpr uint32_t tc_ring(int stages) {
+  return 2 * kTcStage * (uint32_t)stages > kTcTile ? 2 * kTcStage * (uint32_t)stages : (kTcTile + 63) / 64 * 64;
+}
+__host__ __device__ constexpr int tc_smem(int stages) { return (int)tc_ring(stages) + 1024 + 128; }
+static_assert(4 * tc_smem(kTcWStages) > 227 * 1024, "four CTAs per SM would oversubscribe tensor memory");
 
 // byte offset of element (row, k) of a 128 x 64 BF16 chunk: core matrix
 // (row / 8, k / 8) at ((row / 8) * 8 + k / 8) * 128, row % 8 at 16-byte steps,
@@ -67,110 +87,300 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity) {
   return false;
 }
 
-// op(A) element (r, k): tA ? A[k M + r] : A[r K + k]; op(B) element (k, n):
-// tB ? B[n K + k] : (Bb ? Bb[k N + n] : B[k N + n]).
-__global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                             const __nv_bfloat16* __restrict__ Bb,
-                                                             float* __restrict__ C, const float* __restrict__ bias,
-                                                             int M, int N, int K, int tA, int tB,
-                                                             int* __restrict__ err) {
-  extern __shared__ unsigned char tc_smem_raw[];
-  const uint32_t raw = (uint32_t)__cvta_generic_to_shared(tc_smem_raw);
-  const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
-  unsigned char* sA = tc_smem_raw + pad;
-  unsigned char* sB = sA + kTcStage;
-  const uint32_t aS = raw + pad, bS = aS + kTcStage, mS = bS + kTcStage, tS = mS + 8;
-  const uint32_t* tslot = reinterpret_cast<const uint32_t*>(sB + kTcStage + 8);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * kTcM, n0 = blockIdx.x * kTcN;
+// One CTA's tensor memory (128 columns), ring of operand chunks and mbarriers
+// (one per chunk slot).
+struct TcCta {
+  unsigned char* ring;
+  uint32_t ringS, mS, tmem;
+  int stages;
 
-  if (warp == 0) {  // whole warp: 128 columns of tensor memory, address written to tslot
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tS), "r"(kTcN));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mS));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tslot;
-
-  bool ok = true;
-  int cfail = 0;
-  const int nchunk = (K + kTcK - 1) / kTcK;
-  for (int c = 0; c < nchunk; ++c) {
-    const int k0 = c * kTcK;
-    // stage the chunk (zero outside M, N, K); the previous chunk's MMAs are done
-    for (int x = tid; x < kTcM * kTcK; x += kTcThreads) {
-      const int r = tA ? x % kTcM : x / kTcK, k = tA ? x / kTcM : x % kTcK;
-      const int gr = m0 + r, gk = k0 + k;
-      float a = 0.0f;
-      if (gr < M && gk < K) a = tA ? A[(size_t)gk * M + gr] : A[(size_t)gr * K + gk];
-      *reinterpret_cast<__nv_bfloat16*>(sA + tc_off(r, k)) = __float2bfloat16(a);
+  __device__ __forceinline__ void init(unsigned char* raw_ptr, int nstages) {
+    stages = nstages;
+    const uint32_t raw = (uint32_t)__cvta_generic_to_shared(raw_ptr);
+    const uint32_t pad = (1024u - (raw & 1023u)) & 1023u;
+    ring = raw_ptr + pad;
+    ringS = raw + pad;
+    mS = ringS + tc_ring(nstages);
+    const uint32_t tS = mS + 64;
+    if (threadIdx.x < 32) {  // whole warp: 128 columns of tensor memory, address written to tS
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tS), "r"(kTcN));
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    for (int x = tid; x < kTcN * kTcK; x += kTcThreads) {
-      const int n = tB ? x / kTcK : x % kTcN, k = tB ? x % kTcK : x / kTcN;
-      const int gn = n0 + n, gk = k0 + k;
-      __nv_bfloat16 v = __float2bfloat16(0.0f);
-      if (gn < N && gk < K)
-        v = tB ? __float2bfloat16(B[(size_t)gn * K + gk])
-               : (Bb ? Bb[(size_t)gk * N + gn] : __float2bfloat16(B[(size_t)gk * N + gn]));
-      *reinterpret_cast<__nv_bfloat16*>(sB + tc_off(n, k)) = v;
+    if (threadIdx.x == 0) {
+      for (int i = 0; i < nstages; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mS + 8 * i));
+      asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    // generic-proxy stores become visible to the tensor cores' (async proxy) reads
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-      for (int kk = 0; kk < kTcK / 16; ++kk) {
-        if (k0 + kk * 16 >= K) break;  // the zero padding past K needs no MMA (kk = 0 always runs)
-        const uint64_t ad = tc_desc(aS + (uint32_t)kk * 256u, kTcLbo, kTcSbo);
-        const uint64_t bd = tc_desc(bS + (uint32_t)kk * 256u, kTcLbo, kTcSbo);
-        const uint32_t accum = (c > 0 || kk > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(kTcIdesc), "r"(accum));
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mS)
-                   : "memory");
-    }
-    ok = tc_wait(mS, (uint32_t)(c & 1));
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (__syncthreads_or(!ok)) {
-      ok = false;
-      cfail = c;
-      break;
-    }
+    tmem = *reinterpret_cast<const uint32_t*>(ring + tc_ring(nstages) + 64);
   }
-  if (ok) {
-#pragma unroll 1
-    for (int c0 = 0; c0 < kTcN; c0 += 8) {
-      uint32_t v[8];
+  __device__ __forceinline__ uint32_t chunk(int c) const { return (uint32_t)(c % stages) * 2 * kTcStage; }
+
+  // one thread: the MMAs of chunk c (k0 = 64 c; the zero padding past K needs none)
+  __device__ __forceinline__ void mma(int c, int K) const {
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t aS = ringS + chunk(c), bS = aS + kTcStage;
+#pragma unroll
+    for (int kk = 0; kk < kTcK / 16; ++kk) {
+      if (c * kTcK + kk * 16 >= K) break;
+      const uint64_t ad = tc_desc(aS + (uint32_t)kk * 256u, kTcLbo, kTcSbo);
+      const uint64_t bd = tc_desc(bS + (uint32_t)kk * 256u, kTcLbo, kTcSbo);
+      const uint32_t accum = (c > 0 || kk > 0) ? 1u : 0u;
       asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+          "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+          "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+          "l"(ad), "l"(bd), "r"(kTcIdesc), "r"(accum));
+    }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                     mS + 8 * (c % stages))
+                 : "memory");
+  }
+  // chunk c's MMAs (and all before them) are done
+  __device__ __forceinline__ bool wait(int c) const {
+    const bool ok = tc_wait(mS + 8 * (c % stages), (uint32_t)((c / stages) & 1));
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    return ok;
+  }
+  // the accumulator as a row-major FP32 tile in the ring; every thread, all MMAs done
+  __device__ __forceinline__ float* tile() const {
+    float* t = reinterpret_cast<float*>(ring);
+    const int warp = threadIdx.x >> 5;
+#pragma unroll 1
+    for (int c0 = 0; c0 < kTcN; c0 += 16) {
+      uint32_t v[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+          "%15}, [%16];\n"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
           : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      const int r = m0 + warp * 32 + lane;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int col = n0 + c0 + j;
-        if (r < M && col < N) C[(size_t)r * N + col] = __uint_as_float(v[j]) + (bias ? bias[col] : 0.0f);
+      for (int j = 0; j < 16; ++j) t[threadIdx.x * kTcTileLd + c0 + j] = __uint_as_float(v[j]);
+    }
+    __syncthreads();
+    return t;
+  }
+  __device__ __forceinline__ void release() const {
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (threadIdx.x < 32)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcN));
+  }
+  // a chunk's MMAs did not complete in time: one more bounded wait before the
+  // tensor memory they write is released
+  __device__ __forceinline__ void give_up(int c, int* err) const {
+    wait(c);
+    if (threadIdx.x == 0) atomicExch(err, 1);
+  }
+};
+
+__device__ __forceinline__ float tc_sig(float z) { return 1.0f / (1.0f + expf(-z)); }
+
+// rows of the next GEMM's operands: whole 64-element chunks
+__host__ __device__ constexpr int tc_ld(int k) { return (k + kTcK - 1) / kTcK * kTcK; }
+
+// Epilogue of a layer.  M rows (batch), N columns; ldo = tc_ld(N).
+struct TcEpi {
+  const float* bias;    // kTcHidden, kTcOut, kTcLoss: [N]
+  float* Z;             // kTcHidden out, kTcBack in: pre-activations [M x N]
+  __nv_bfloat16* O;     // kTcHidden: silu(z); kTcLoss, kTcBack: the gradient; [M x ldo], padding written as zero
+  float* Y;             // kTcOut: [M x N]
+  const float *t, *mask;  // kTcLoss: [M x N]
+  const float* scal;    // kTcLoss: [1] = sum of the mask
+  float* colsum;        // kTcLoss, kTcBack: this row tile's column sums of the gradient, [row tile][cs_ld]
+  int cs_ld;
+  float* lossp;         // kTcLoss: this CTA's part of the loss numerator
+};
+enum { kTcHidden, kTcOut, kTcLoss, kTcBack };
+
+// C[M x N] = A[M x K] B[N x K]^T: A, B BF16, K-contiguous, row strides tc_ld(K).
+template <int EPI>
+__global__ void __launch_bounds__(kTcThreads) tc_layer_kernel(const __nv_bfloat16* __restrict__ A,
+                                                              const __nv_bfloat16* __restrict__ B, int M, int N,
+                                                              int K, TcEpi e, int* __restrict__ err) {
+  extern __shared__ unsigned char tc_smem_raw[];
+  TcCta T;
+  T.init(tc_smem_raw, kTcStages);
+  const int tid = threadIdx.x;
+  const int m0 = blockIdx.y * kTcM, n0 = blockIdx.x * kTcN;
+  const int ld = tc_ld(K), nchunk = ld / kTcK;
+  auto load = [&](int c) {  // 16-byte units of chunk c, rows past M or N zero-filled
+    if (c < nchunk) {
+      const uint32_t base = T.ringS + T.chunk(c);
+#pragma unroll
+      for (int i = 0; i < kTcM * kTcK / 8 / kTcThreads; ++i) {
+        const int x = tid + i * kTcThreads, r = x >> 3, u = (x & 7) * 8;
+        const bool va = m0 + r < M, vb = n0 + r < N;
+        const __nv_bfloat16* pa = A + (size_t)(va ? m0 + r : 0) * ld + c * kTcK + u;
+        const __nv_bfloat16* pb = B + (size_t)(vb ? n0 + r : 0) * ld + c * kTcK + u;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(base + tc_off(r, u)), "l"(pa),
+                     "r"(va ? 16 : 0)
+                     : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(base + kTcStage + tc_off(r, u)), "l"(pb),
+                     "r"(vb ? 16 : 0)
+                     : "memory");
       }
     }
-  } else {
-    // a chunk's MMAs did not complete in time: give them one more bounded wait
-    // before the tensor memory they write is released
-    tc_wait(mS, (uint32_t)(cfail & 1));
-    if (tid == 0) atomicExch(err, 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int c = 0; c < kTcStages - 1; ++c) load(c);
+  bool ok = true;
+  int cfail = 0;
+  for (int c = 0; c < nchunk; ++c) {
+    // the slot of chunk c + kTcStages - 1 held chunk c - 1
+    if (c > 0 && c + kTcStages - 1 < nchunk) ok = T.wait(c - 1);
+    if (ok) load(c + kTcStages - 1);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kTcStages - 1) : "memory");
+    // the copies become visible to the tensor cores' (async proxy) reads
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      cfail = c - 1;
+      break;
+    }
+    if (tid == 0) T.mma(c, K);
   }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcN));
+  if (ok) {
+    ok = T.wait(nchunk - 1);
+    cfail = nchunk - 1;
+    ok = !__syncthreads_or(!ok);
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (ok) {
+    const float* tile = T.tile();
+    const int col = n0 + tid, rows = M - m0 < kTcM ? M - m0 : kTcM;
+    const int ldo = tc_ld(N);
+    const bool in = col < N;
+    const float b = (EPI != kTcBack && in) ? e.bias[col] : 0.0f;
+    const float inv = EPI == kTcLoss ? 1.0f / fmaxf(e.scal[1], 1.0f) : 0.0f;
+    float sum = 0.0f, num = 0.0f;
+    if (in) {
+#pragma unroll 8
+      for (int r = 0; r < rows; ++r) {
+        const float acc = tile[r * kTcTileLd + tid];
+        const size_t at = (size_t)(m0 + r) * N + col, ao = (size_t)(m0 + r) * ldo + col;
+        if constexpr (EPI == kTcHidden) {
+          const float z = acc + b;
+          e.Z[at] = z;
+          e.O[ao] = __float2bfloat16(z * tc_sig(z));
+        } else if constexpr (EPI == kTcOut) {
+          e.Y[at] = acc + b;
+        } else if constexpr (EPI == kTcLoss) {
+          // loss numerator, dy = 2 mask (y - t) / sum(mask)
+          const float m = e.mask[at], d = (acc + b) - e.t[at];
+          num += m * d * d;
+          const float dy = 2.0f * m * d * inv;
+          sum += dy;
+          e.O[ao] = __float2bfloat16(dy);
+        } else {
+          const float z = e.Z[at], s = tc_sig(z);
+          const float d = acc * (s * (1.0f + z * (1.0f - s)));
+          sum += d;
+          e.O[ao] = __float2bfloat16(d);
+        }
+      }
+    } else if (EPI != kTcOut && col < ldo) {
+      for (int r = 0; r < rows; ++r) e.O[(size_t)(m0 + r) * ldo + col] = __float2bfloat16(0.0f);
+    }
+    if (EPI == kTcLoss || EPI == kTcBack)
+      if (in) e.colsum[(size_t)blockIdx.y * e.cs_ld + col] = sum;
+    if constexpr (EPI == kTcLoss) {
+      __syncthreads();  // the tile has been read
+      float* red = reinterpret_cast<float*>(T.ring);
+      red[tid] = num;
+      __syncthreads();
+      for (int o = kTcThreads / 2; o > 0; o >>= 1) {
+        if (tid < o) red[tid] += red[tid + o];
+        __syncthreads();
+      }
+      if (tid == 0) e.lossp[blockIdx.y * gridDim.x + blockIdx.x] = red[0];
+    }
+  } else {
+    T.give_up(cfail < 0 ? 0 : cfail, err);
+  }
+  T.release();
+}
+
+// One layer's weight gradient G[M x N] = A^T B over the batch: A [batch x lda],
+// B [batch x ldb] BF16; tiles of the launch from tile0 on, tn of them per row
+// of tiles; the product lands at off in a workspace slice.
+struct TcWLayer {
+  const __nv_bfloat16 *A, *B;
+  int lda, ldb, M, N, tn, tile0;
+  size_t off;
+};
+struct TcWgrad {
+  TcWLayer l[3];
+  float* part;   // [split][np]
+  size_t np;
+  int batch, rows;  // batch rows per split (a multiple of 64)
+};
+
+__global__ void __launch_bounds__(kTcThreads) tc_wgrad_kernel(TcWgrad P, int* __restrict__ err) {
+  extern __shared__ unsigned char tc_smem_raw[];
+  TcCta T;
+  T.init(tc_smem_raw, kTcWStages);
+  const int tid = threadIdx.x;
+  int li = 0;
+  while (li < 2 && (int)blockIdx.x >= P.l[li + 1].tile0) ++li;
+  const TcWLayer L = P.l[li];
+  const int tile = blockIdx.x - L.tile0, m0 = tile / L.tn * kTcM, n0 = tile % L.tn * kTcN;
+  const int k_lo = blockIdx.y * P.rows, k_hi = min(k_lo + P.rows, P.batch), K = k_hi - k_lo;
+  const int nchunk = (K + kTcK - 1) / kTcK;
+  // 16-byte units (8 batch rows) of two adjacent columns per thread and step
+  auto stage = [&](const __nv_bfloat16* src, int ld, int c0, int k0, unsigned char* dst) {
+#pragma unroll
+    for (int i = 0; i < kTcM / 2 * (kTcK / 8) / kTcThreads; ++i) {
+      const int x = tid + i * kTcThreads, m = (x & 63) * 2, u = (x >> 6) * 8;
+      uint32_t w[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int k = k0 + u + r;
+        w[r] = (k < k_hi && c0 + m < ld) ? *reinterpret_cast<const uint32_t*>(src + (size_t)k * ld + c0 + m) : 0u;
+      }
+      uint4 lo, hi;
+      lo.x = __byte_perm(w[0], w[1], 0x5410); hi.x = __byte_perm(w[0], w[1], 0x7632);
+      lo.y = __byte_perm(w[2], w[3], 0x5410); hi.y = __byte_perm(w[2], w[3], 0x7632);
+      lo.z = __byte_perm(w[4], w[5], 0x5410); hi.z = __byte_perm(w[4], w[5], 0x7632);
+      lo.w = __byte_perm(w[6], w[7], 0x5410); hi.w = __byte_perm(w[6], w[7], 0x7632);
+      *reinterpret_cast<uint4*>(dst + tc_off(m, u)) = lo;
+      *reinterpret_cast<uint4*>(dst + tc_off(m + 1, u)) = hi;
+    }
+  };
+  bool ok = true;
+  int cfail = 0;
+  for (int c = 0; c < nchunk; ++c) {
+    if (c >= kTcWStages) ok = T.wait(c - kTcWStages);
+    if (ok) {
+      unsigned char* s = T.ring + T.chunk(c);
+      stage(L.A, L.lda, m0, k_lo + c * kTcK, s);
+      stage(L.B, L.ldb, n0, k_lo + c * kTcK, s + kTcStage);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (__syncthreads_or(!ok)) {
+      ok = false;
+      cfail = c - kTcWStages;
+      break;
+    }
+    if (tid == 0) T.mma(c, K);
+  }
+  if (ok) {
+    ok = T.wait(nchunk - 1);
+    cfail = nchunk - 1;
+    ok = !__syncthreads_or(!ok);
+  }
+  if (ok) {
+    const float* t = T.tile();
+    float* out = P.part + (size_t)blockIdx.y * P.np + L.off;
+    const int rows = min(L.M - m0, kTcM);
+    if (n0 + tid < L.N)
+      for (int r = 0; r < rows; ++r) out[(size_t)(m0 + r) * L.N + n0 + tid] = t[r * kTcTileLd + tid];
+  } else {
+    T.give_up(cfail < 0 ? 0 : cfail, err);
+  }
+  T.release();
 }
 
 }  // namespace fsim
