@@ -215,14 +215,14 @@ cudaError_t pack(const fsim_mlp* n, cudaStream_t s) {
 __global__ void prep_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ xb, int b, int nin,
                             const float* __restrict__ mask, size_t nmask, float* __restrict__ scal) {
   const int ld = tc_ld(nin);
-  const size_t n = (size_t)b * ld, step = (size_t)gridDim.x * blockDim.x;
-  const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  for (size_t i = i0; i < n; i += step) {
-    const int c = (int)(i % ld);
-    xb[i] = __float2bfloat16(c < nin ? x[i / ld * nin + c] : 0.0f);
-  }
+  const size_t step = (size_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  // a warp per row and step
+  for (size_t r = i0 / 32; r < (size_t)b; r += step / 32)
+    for (int c = threadIdx.x & 31; c < ld; c += 32)
+      xb[r * ld + c] = __float2bfloat16(c < nin ? x[r * nin + c] : 0.0f);
   if (!mask) return;
   float s = 0.0f;
+#pragma unroll 4
   for (size_t i = i0; i < nmask; i += step) s += mask[i];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) atomicAdd(scal + 1, s);

@@ -1,15 +1,16 @@
 // BF16 x BF16 -> FP32 GEMMs on the fifth-generation tensor cores for the
 // learned-guess network, with its element-wise steps as epilogues.
 //
-// One CTA of four warps per 128 x 128 tile of the product.  The K dimension is
+// One CTA of eight warps per 128 x 128 tile of the product.  The K dimension is
 // walked in chunks of 64, each staged into shared memory in the canonical
 // no-swizzle K-major layout (core matrices of 8 rows x 16 bytes, 128 contiguous
 // bytes each); one thread issues four tcgen05.mma (M 128, N 128, K 16 each)
 // that accumulate in tensor memory (128 lanes x 128 FP32 columns) and commits
 // them to the chunk's mbarrier.  Then the accumulator goes through shared
 // memory (tcgen05.ld gives a thread one row; the epilogue wants a column) and
-// thread t runs the epilogue on column t of the tile, row by row: global
-// accesses coalesce and a column sum is one register.  A wait that runs out
+// threads t and t + 128 run the epilogue on the halves of column t of the tile,
+// eight rows' inputs in flight: global accesses coalesce and a column sum is
+// one register.  A wait that runs out
 // sets *err and the CTA frees its tensor memory and returns.
 //
 //  * tc_layer_kernel: forward layers and the data gradients.  Both operands lie
@@ -33,7 +34,7 @@
 namespace fsim {
 
 constexpr int kTcM = 128, kTcN = 128, kTcK = 64;
-constexpr int kTcThreads = 128;
+constexpr int kTcThreads = 256;
 constexpr uint32_t kTcStage = (uint32_t)kTcM * kTcK * 2;  // bytes of one operand chunk
 constexpr int kTcStages = 4;                      // chunks in flight, layers
 constexpr int kTcWStages = 2;                     // chunks in flight, weight gradients
@@ -145,9 +146,10 @@ struct TcCta {
   // the accumulator as a row-major FP32 tile in the ring; every thread, all MMAs done
   __device__ __forceinline__ float* tile() const {
     float* t = reinterpret_cast<float*>(ring);
-    const int warp = threadIdx.x >> 5;
+    const int warp = (threadIdx.x >> 5) & 3, half = threadIdx.x >> 7;  // warps w and w + 4: rows 32w .. 32w + 31
+    const int row = threadIdx.x & 127;
 #pragma unroll 1
-    for (int c0 = 0; c0 < kTcN; c0 += 16) {
+    for (int c0 = half * (kTcN / 2); c0 < (half + 1) * (kTcN / 2); c0 += 16) {
       uint32_t v[16];
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -157,7 +159,7 @@ struct TcCta {
           : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-      for (int j = 0; j < 16; ++j) t[threadIdx.x * kTcTileLd + c0 + j] = __uint_as_float(v[j]);
+      for (int j = 0; j < 16; ++j) t[row * kTcTileLd + c0 + j] = __uint_as_float(v[j]);
     }
     __syncthreads();
     return t;
@@ -249,53 +251,67 @@ __global__ void __launch_bounds__(kTcThreads) tc_layer_kernel(const __nv_bfloat1
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   if (ok) {
-    const float* tile = T.tile();
-    const int col = n0 + tid, rows = M - m0 < kTcM ? M - m0 : kTcM;
+    float* tile = T.tile();
+    const int tc = tid & 127, col = n0 + tc;
+    const int r0 = (tid >> 7) * (kTcM / 2), r1 = min(r0 + kTcM / 2, M - m0);
     const int ldo = tc_ld(N);
     const bool in = col < N;
     const float b = (EPI != kTcBack && in) ? e.bias[col] : 0.0f;
     const float inv = EPI == kTcLoss ? 1.0f / fmaxf(e.scal[1], 1.0f) : 0.0f;
     float sum = 0.0f, num = 0.0f;
     if (in) {
-#pragma unroll 8
-      for (int r = 0; r < rows; ++r) {
-        const float acc = tile[r * kTcTileLd + tid];
-        const size_t at = (size_t)(m0 + r) * N + col, ao = (size_t)(m0 + r) * ldo + col;
-        if constexpr (EPI == kTcHidden) {
-          const float z = acc + b;
-          e.Z[at] = z;
-          e.O[ao] = __float2bfloat16(z * tc_sig(z));
-        } else if constexpr (EPI == kTcOut) {
-          e.Y[at] = acc + b;
-        } else if constexpr (EPI == kTcLoss) {
-          // loss numerator, dy = 2 mask (y - t) / sum(mask)
-          const float m = e.mask[at], d = (acc + b) - e.t[at];
-          num += m * d * d;
-          const float dy = 2.0f * m * d * inv;
-          sum += dy;
-          e.O[ao] = __float2bfloat16(dy);
-        } else {
-          const float z = e.Z[at], s = tc_sig(z);
-          const float d = acc * (s * (1.0f + z * (1.0f - s)));
-          sum += d;
-          e.O[ao] = __float2bfloat16(d);
+      for (int r = r0; r < r1; r += 8) {
+        float p[8], q[8];  // inputs of eight rows, all loads in flight
+        if constexpr (EPI == kTcBack || EPI == kTcLoss) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const size_t at = (size_t)(m0 + min(r + u, r1 - 1)) * N + col;
+            p[u] = EPI == kTcBack ? e.Z[at] : e.mask[at];
+            if constexpr (EPI == kTcLoss) q[u] = e.t[at];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          if (r + u >= r1) break;
+          const float acc = tile[(r + u) * kTcTileLd + tc];
+          const size_t at = (size_t)(m0 + r + u) * N + col, ao = (size_t)(m0 + r + u) * ldo + col;
+          if constexpr (EPI == kTcHidden) {
+            const float z = acc + b;
+            e.Z[at] = z;
+            e.O[ao] = __float2bfloat16(z * tc_sig(z));
+          } else if constexpr (EPI == kTcOut) {
+            e.Y[at] = acc + b;
+          } else if constexpr (EPI == kTcLoss) {
+            // loss numerator, dy = 2 mask (y - t) / sum(mask)
+            const float d = (acc + b) - q[u];
+            num += p[u] * d * d;
+            const float dy = 2.0f * p[u] * d * inv;
+            sum += dy;
+            e.O[ao] = __float2bfloat16(dy);
+          } else {
+            const float z = p[u], s = tc_sig(z);
+            const float d = acc * (s * (1.0f + z * (1.0f - s)));
+            sum += d;
+            e.O[ao] = __float2bfloat16(d);
+          }
         }
       }
     } else if (EPI != kTcOut && col < ldo) {
-      for (int r = 0; r < rows; ++r) e.O[(size_t)(m0 + r) * ldo + col] = __float2bfloat16(0.0f);
+      for (int r = r0; r < r1; ++r) e.O[(size_t)(m0 + r) * ldo + col] = __float2bfloat16(0.0f);
     }
-    if (EPI == kTcLoss || EPI == kTcBack)
-      if (in) e.colsum[(size_t)blockIdx.y * e.cs_ld + col] = sum;
-    if constexpr (EPI == kTcLoss) {
+    if constexpr (EPI == kTcLoss || EPI == kTcBack) {
       __syncthreads();  // the tile has been read
-      float* red = reinterpret_cast<float*>(T.ring);
-      red[tid] = num;
+      tile[tid] = sum;
+      tile[kTcThreads + tid] = num;
       __syncthreads();
-      for (int o = kTcThreads / 2; o > 0; o >>= 1) {
-        if (tid < o) red[tid] += red[tid + o];
-        __syncthreads();
+      if (tid < kTcN && in) e.colsum[(size_t)blockIdx.y * e.cs_ld + col] = tile[tid] + tile[tid + kTcN];
+      if constexpr (EPI == kTcLoss) {
+        for (int o = kTcThreads / 2; o > 0; o >>= 1) {
+          if (tid < o) tile[kTcThreads + tid] += tile[kTcThreads + tid + o];
+          __syncthreads();
+        }
+        if (tid == 0) e.lossp[blockIdx.y * gridDim.x + blockIdx.x] = tile[kTcThreads];
       }
-      if (tid == 0) e.lossp[blockIdx.y * gridDim.x + blockIdx.x] = red[0];
     }
   } else {
     T.give_up(cfail < 0 ? 0 : cfail, err);
@@ -374,9 +390,10 @@ __global__ void __launch_bounds__(kTcThreads) tc_wgrad_kernel(TcWgrad P, int* __
   if (ok) {
     const float* t = T.tile();
     float* out = P.part + (size_t)blockIdx.y * P.np + L.off;
-    const int rows = min(L.M - m0, kTcM);
-    if (n0 + tid < L.N)
-      for (int r = 0; r < rows; ++r) out[(size_t)(m0 + r) * L.N + n0 + tid] = t[r * kTcTileLd + tid];
+    const int tc = tid & 127, r0 = (tid >> 7) * (kTcM / 2), r1 = min(r0 + kTcM / 2, L.M - m0);
+    if (n0 + tc < L.N)
+#pragma unroll 8
+      for (int r = r0; r < r1; ++r) out[(size_t)(m0 + r) * L.N + n0 + tc] = t[r * kTcTileLd + tc];
   } else {
     T.give_up(cfail < 0 ? 0 : cfail, err);
   }
