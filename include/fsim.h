@@ -215,14 +215,15 @@ int fsim_j_build(fsim_basis* b, const double* D, double* J, const fsim_fock_opts
  * for class pairs with fewer than 2 x 128 x SMs / 9 quartets) and the
  * ket-component chunks shared out over csplit = 1, 2 or 4 warp groups (a CTA
  * of 128 threads takes floor(128 / csplit / psplit) kets), and the
- * warp-cooperative kernel (4 kets per CTA) -- and keeps the fastest in the
- * basis' cached plan, which later fsim_fock_build calls with the same options
- * use.  FSIM_DFLOAT: every shape with the double-float kernel and with the
- * FP64 kernel (both FP64-accurate), no cooperative kernel.  choice (36
- * entries, optional): 10 * psplit + csplit for the unrolled kernel (+ 1000
- * when a double-float build runs the class pair with the FP64 kernel), -1 for
- * the cooperative kernel, 0 for class pairs
- * without work; best_ms (36, optional): its median time.  Index X*6+Y as in
+ * cooperative kernel (a warp per quartet in FP32, a CTA per quartet in FP64) --
+ * and keeps the fastest in the basis' cached plan, which later fsim_fock_build
+ * calls with the same options use.  FSIM_DFLOAT: every shape with the
+ * double-float kernel and with the FP64 kernel (both FP64-accurate), and the
+ * FP64 cooperative kernel where the untuned plan has it.  choice (36 entries,
+ * optional): 10 * psplit + csplit for the unrolled kernel (+ 1000 when a
+ * double-float build runs the class pair with the FP64 kernel), -1 for the
+ * cooperative kernel (FSIM_DFLOAT: 0, as planned), 0 for class pairs without
+ * work; best_ms (36, optional): its median time.  Index X*6+Y as in
  * fsim_last_class_times.
  */
 int fsim_autotune(fsim_basis* b, const fsim_fock_opts* opts, int* choice, float* best_ms);

@@ -117,9 +117,22 @@ __global__ void split4_kernel(const double4_32a* __restrict__ in, dfloat4* __res
 
 // The double-float table keeps e^{-T_i} in its last column (an order no class
 // reaches), read by the double-float Boys function.
-__global__ void boys_exp_column_kernel(dfloat* __restrict__ tab) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kBoysN64; i += gridDim.x * blockDim.x)
-    tab[(size_t)i * kBoysCols + kBoysCols - 1] = dsplit_rn(exp(-i * kBoysH64));
+// Per-order tables of the quartet kernels from the full FP64 table (stage_boys).
+template <typename Real>
+__global__ void boys_orders_kernel(const double* __restrict__ full, Real* __restrict__ out) {
+  constexpr int NC = Boys<Real>::NCOL;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < kBoysOrders * kBoysN64 * NC; x += gridDim.x * blockDim.x) {
+    const int L = x / (kBoysN64 * NC), r = x % (kBoysN64 * NC), c = r % NC;
+    double v = full[(size_t)(r / NC) * kBoysCols + Boys<Real>::col(L, c)];
+    if constexpr (std::is_same<Real, double>::value) {
+      double f = 1.0;
+      if (c < kBoysK64)
+        for (int k = 2; k <= c; ++k) f *= k;
+      out[(size_t)L * kBoysOrderLd + r] = v / f;
+    } else {
+      out[(size_t)L * kBoysOrderLd + r] = dsplit_rn(v);
+    }
+  }
 }
 
 void launch_split(const double* in, dfloat* out, size_t n, cudaStream_t s) {
@@ -137,11 +150,9 @@ int ensure_dfloat(fsim_basis* b) {
     launch_split(C.pd64, C.pdx, nf, 0);
     split4_kernel<<<(unsigned)std::min<size_t>((nq + 255) / 256, 1024), 256>>>(C.pq64, C.pqx, nq);
   }
-  const size_t nb = (size_t)kBoysN64 * kBoysCols;
   if (!b->d_boysx) {
-    FSIM_TRY(dev_alloc(&b->d_boysx, nb));
-    launch_split(b->d_boys64, b->d_boysx, nb, 0);
-    boys_exp_column_kernel<<<(kBoysN64 + 127) / 128, 128>>>(b->d_boysx);
+    FSIM_TRY(dev_alloc(&b->d_boysx, (size_t)kBoysOrders * kBoysOrderLd));
+    boys_orders_kernel<dfloat><<<128, 256>>>(b->d_boys64, b->d_boysx);
   }
   if (!b->d_Dx) FSIM_TRY(dev_alloc(&b->d_Dx, (size_t)b->nbf * b->nbf));
   FSIM_CK(cudaGetLastError());
@@ -407,10 +418,14 @@ int fsim_basis_create_ex(const fsim_atom* atoms, int natom, const fsim_shell_des
   {
     std::vector<double> t64, t32d;
     boys_table(t64, kBoysN64, kBoysH64);
+    // last column, beyond every order in use: e^{-T_i}
+    for (int i = 0; i < kBoysN64; ++i) t64[(size_t)i * kBoysCols + kBoysCols - 1] = std::exp(-i * kBoysH64);
     boys_table(t32d, kBoysN32, (double)kBoysH32);
     std::vector<float> t32(t32d.begin(), t32d.end());
     UP(b->d_boys64, t64.data(), t64.size());
     UP(b->d_boys32, t32.data(), t32.size());
+    if ((rc = dev_alloc(&b->d_boys64s, (size_t)kBoysOrders * kBoysOrderLd)) != FSIM_OK) return fail(rc);
+    boys_orders_kernel<double><<<128, 256>>>(b->d_boys64, b->d_boys64s);
   }
 #undef UP
   // canonical pairs per class: higher l first; equal l: higher shell index first
@@ -464,7 +479,7 @@ void fsim_basis_destroy(fsim_basis* b) {
   }
   dev_free(b->d_cen); dev_free(b->d_alpha); dev_free(b->d_coef); dev_free(b->d_nprim);
   dev_free(b->d_l); dev_free(b->d_ao); dev_free(b->d_axyz); dev_free(b->d_Z);
-  dev_free(b->d_boys64); dev_free(b->d_boys32); dev_free(b->d_boysx); dev_free(b->d_Dx);
+  dev_free(b->d_boys64); dev_free(b->d_boys32); dev_free(b->d_boys64s); dev_free(b->d_boysx); dev_free(b->d_Dx);
   dev_free(b->d_Jacc); dev_free(b->d_Kacc); dev_free(b->d_D); dev_free(b->d_J); dev_free(b->d_K);
   dev_free(b->d_D32);
   dev_free(b->d_sti); dev_free(b->d_stc); dev_free(b->d_sci); dev_free(b->d_scc);

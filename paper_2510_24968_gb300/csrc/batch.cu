@@ -215,7 +215,7 @@ int launch_batch(fsim_batch* bt, int prec, cudaStream_t s, bool dry) {
         p.psplit = 1;
         p.csplit = 1;
         p.bra_ppmax = C.bra_ppmax;
-        p.boys = std::is_same<Real, double>::value ? (const Real*)bt->b[0]->d_boys64 : (const Real*)bt->b[0]->d_boys32;
+        p.boys = quartet_boys<Real>(bt->b[0]);
         p.boys64_T = INFINITY;
         e = dispatch<Real>(X, Y, p, s);
       }

@@ -45,6 +45,12 @@ constexpr double kSqrtPi = 1.7724538509055160273;
 // 1/(2n+1) and 1/k as compile-time constants
 __host__ __device__ constexpr double inv_odd(int n) { return 1.0 / (2 * n + 1); }
 __host__ __device__ constexpr double inv_int(int k) { return 1.0 / k; }
+// 1/k!
+__host__ __device__ constexpr double inv_fact(int k) {
+  double r = 1.0;
+  for (int i = 2; i <= k; ++i) r /= i;
+  return r;
+}
 
 // Large-T branch in double: F_0 = sqrt(pi/T)/2, upward recursion.
 template <int L>
@@ -126,9 +132,6 @@ __device__ __forceinline__ void boys_fp32(float T, float (&F)[L + 1], const floa
   }
 }
 
-// 1/k! as a double-float constant
-__host__ __device__ constexpr double inv_fact(int k) { return k <= 1 ? 1.0 : inv_fact(k - 1) / k; }
-
 // Double-float Boys function without FP64 operations.  `row` holds, for the
 // nearest grid point T_i, F_{L..L+K-1}(T_i) and in slot K the value e^{-T_i}.
 //  * T < 36: Taylor sum for F_L as in FP64; e^{-T} = e^{-T_i} e^{x},
@@ -180,13 +183,73 @@ __device__ __forceinline__ void boys_dfloat(dfloat T, dfloat (&F)[L + 1], const 
   }
 }
 
+// x^{-1/2} for normal x > 0: the hardware estimate y (about 20 correct bits)
+// times the series of (1 - e)^{-1/2}, e = 1 - x y^2, to e^2 (next term < 2^-58):
+// five FP64 operations and no special-case branch.
+__device__ __forceinline__ double rsqrt_fp64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// F_0..F_L in FP64 from u = -2T, for kernels whose time is the number of FP64
+// instructions (two per clock and SM on GB300).  `row i` of tabL holds, for
+// T_i = i / 16, F_{L..L+K-1}(T_i) / k! in slots k < K and e^{-T_i} in slot
+// `ecol` (SCALED; unscaled F_{L+k} otherwise).
+//  * T_i: adding 3 2^47 rounds T to a multiple of its last place, 1/16, and
+//    leaves i in the low word: no conversions; range check on the high word.
+//  * e^{-T} = e^{-T_i} e^{x}, |x| <= 1/32, Taylor to x^7 (next term < 2^-55),
+//    in place of the library exponential.
+//  * T >= 36: F_0 from rsqrt_fp64.  e^{-T} <= 2.4e-16; taken from FP32 (2e-6 of
+//    it, mostly from rounding T) it leaves 1e-16 of F_5 at T = 36 and less of
+//    lower orders; from order 6 on it is the FP64 exponential.
+// One (ps|ss) primitive quartet went from 67 to about 46 FP64 instructions with
+// this and rsqrt_fp64 (ncu: pipe share times duration).
+template <int K>
+constexpr double inv_fact_c = inv_fact(K);  // a constant in device code too, never a call
+constexpr double kBoysRound = 422212465065984.0;  // 3 2^47
+template <int L, bool SCALED>
+__device__ __forceinline__ void boys_fp64_u(double u, double (&F)[L + 1], const double* __restrict__ tabL, int stride,
+                                            int ecol) {
+  if (__double2hiint(u) < (int)0xC0520000) {  // as integers, for u <= 0: -u < 72
+    const double t = fma(u, -0.5, kBoysRound);
+    const double Ti = t - kBoysRound;
+    const double x = fma(u, 0.5, Ti);  // -(T - T_i)
+    const double* row = tabL + __double2loint(t) * stride;
+    double acc = row[kBoysK64 - 1];
+#pragma unroll
+    for (int k = kBoysK64 - 1; k >= 1; --k) acc = fma(acc, SCALED ? x : x * inv_int(k), row[k - 1]);
+    F[L] = acc;
+    if constexpr (L > 0) {
+      constexpr int kExpTerms = 7;
+      double ex = inv_fact_c<kExpTerms>;
+      static_for<kExpTerms>([&](auto I) { ex = fma(ex, x, inv_fact_c<kExpTerms - 1 - decltype(I)::value>); });
+      const double e = row[ecol] * ex;
+#pragma unroll
+      for (int n = L - 1; n >= 0; --n) F[n] = n > 0 ? fma(-u, F[n + 1], e) * inv_odd(n) : fma(-u, F[1], e);
+    }
+  } else {
+    const double rs = rsqrt_fp64(-0.5 * u);
+    F[0] = 0.5 * kSqrtPi * rs;
+    if constexpr (L > 0) {
+      const double h = 0.5 * rs * rs, e = L <= 5 ? (double)expf(0.5f * (float)u) : exp(0.5 * u);
+#pragma unroll
+      for (int n = 1; n <= L; ++n) F[n] = ((2 * n - 1) * F[n - 1] - e) * h;
+    }
+  }
+}
+
 template <typename Real>
 struct Boys;
 template <>
 struct Boys<double> {
-  static constexpr int K = kBoysK64, NROW = kBoysN64, NCOL = K;
-  // table column staged in slot c (of NCOL) for class order L
-  static __host__ __device__ constexpr int col(int L, int c) { return L + c; }
+  // slots 0..K-1: F_{L+k} / k!; slot K: e^{-T_i}, kept in the table's last
+  // column, which no class order reaches (L + K - 1 <= 19 < kBoysCols - 1)
+  static constexpr int K = kBoysK64, NROW = kBoysN64, NCOL = K + 1;
+  // table column in slot c (of NCOL) for class order L
+  static __host__ __device__ constexpr int col(int L, int c) { return c < K ? L + c : kBoysCols - 1; }
+  // from the full table (unscaled, rows of kBoysCols)
   template <int L>
   static __device__ __forceinline__ void eval(double T, double (&F)[L + 1], const double* tabL, int stride,
                                               float /*t64*/) {
@@ -217,5 +280,26 @@ struct Boys<dfloat> {
     boys_dfloat<L>(T, F, tabL, stride);
   }
 };
+
+// The quartet kernels' tables in global memory.  FP64 and double-float: one
+// block of kBoysOrderLd values per class order L = 0..8, in the staged layout
+// ([row][slot], F_{L+k}/k! in FP64), so that a CTA's prologue is 16-byte
+// copies; FP32: the full table, columns picked while staging (5 KB).
+constexpr int kBoysOrders = 9;
+constexpr int kBoysOrderLd = (kBoysN64 * (kBoysK64 + 1) + 1) / 2 * 2;
+
+template <typename Real, int L>
+__device__ __forceinline__ void stage_boys(Real* __restrict__ dst, const Real* __restrict__ tab) {
+  constexpr int BK = Boys<Real>::NCOL, BR = Boys<Real>::NROW;
+  if constexpr (sizeof(Real) == 8) {
+    static_assert(BR == kBoysN64 && BK == kBoysK64 + 1 && L < kBoysOrders, "staged layout");
+    const uint4* src = reinterpret_cast<const uint4*>(tab + (size_t)L * kBoysOrderLd);
+#pragma unroll 8
+    for (int x = threadIdx.x; x < kBoysOrderLd / 2; x += blockDim.x) reinterpret_cast<uint4*>(dst)[x] = __ldg(src + x);
+  } else {
+    for (int x = threadIdx.x; x < BR * BK; x += blockDim.x)
+      dst[x] = tab[(x / BK) * kBoysCols + Boys<Real>::col(L, x % BK)];
+  }
+}
 
 }  // namespace fsim

@@ -140,6 +140,40 @@ __device__ __forceinline__ float rsqrt_r<float>(float x) { return rsqrtf(x); }
 template <>
 __device__ __forceinline__ dfloat rsqrt_r<dfloat>(dfloat x) { return rsqrt_dfloat(x); }
 
+// Source terms R^n_000 = (-2 al)^n F_n(al |P - Q|^2) / sqrt(p + q), n <= L, of
+// one primitive quartet (al = p q / (p + q), X.. = P - Q).  boysL: staged table.
+template <typename Real, int L>
+__device__ __forceinline__ void prim_sources(Real p, Real q, Real X, Real Y, Real Z, Real (&src)[L + 1],
+                                             const Real* __restrict__ boysL, int bstride, float t64) {
+  const Real s = p + q;
+  if constexpr (std::is_same<Real, double>::value) {
+    const double rs = rsqrt_fp64(s);
+    const double m2a = -2.0 * p * q * (rs * rs);
+    double F[L + 1];
+    boys_fp64_u<L, true>(m2a * (X * X + Y * Y + Z * Z), F, boysL, bstride, kBoysK64);
+    double fac = rs;
+    src[0] = fac * F[0];
+#pragma unroll
+    for (int n = 1; n <= L; ++n) {
+      fac *= m2a;
+      src[n] = fac * F[n];
+    }
+  } else {
+    const Real rs = rsqrt_r<Real>(s);
+    const Real al = p * q * (rs * rs);
+    const Real T = al * (X * X + Y * Y + Z * Z);
+    Real F[L + 1];
+    Boys<Real>::template eval<L>(T, F, boysL, bstride, t64);
+    Real fac = rs;
+    const Real m2a = Real(-2) * al;
+#pragma unroll
+    for (int n = 0; n <= L; ++n) {
+      src[n] = fac * F[n];
+      fac *= m2a;
+    }
+  }
+}
+
 // Chunk bookkeeping for the ket side: chunks of CS consecutive components, the
 // last one possibly shorter.
 template <class KC, int CS>
@@ -197,21 +231,9 @@ __device__ __forceinline__ void quartet_chunk(Real* __restrict__ so, const BraAt
       const Real* kp = ket.pd + (size_t)k * ket.n + j;
       const auto q4 = ket.pq[(size_t)k * ket.n + j];
       const Real q = q4.x, Qx = q4.y, Qy = q4.z, Qz = q4.w;
-      const Real s = p + q;
-      const Real rs = rsqrt_r<Real>(s);
-      const Real al = p * q * (rs * rs);
       const Real X = Px - Qx, Y = Py - Qy, Z = Pz - Qz;
-      const Real T = al * (X * X + Y * Y + Z * Z);
-      Real F[L + 1];
-      Boys<Real>::template eval<L>(T, F, boysL, bstride, t64);
       Real src[L + 1];
-      Real fac = rs;
-      const Real m2a = Real(-2) * al;
-#pragma unroll
-      for (int n = 0; n <= L; ++n) {
-        src[n] = fac * F[n];
-        fac *= m2a;
-      }
+      prim_sources<Real, L>(p, q, X, Y, Z, src, boysL, bstride, t64);
       Real R[NH];
       hermite_R<Real, L>(R, src, X, Y, Z);
       Real Ek[NZM];
@@ -304,7 +326,7 @@ __device__ __forceinline__ int find_bra(const int* __restrict__ prefix, int n, i
 // symmetrises J = (J_acc + J_acc^T)/4 and K = (K_acc + K_acc^T)/8.
 template <typename Real>
 __host__ __device__ constexpr size_t jk_boys_smem() {
-  return (size_t)Boys<Real>::NROW * Boys<Real>::NCOL * sizeof(Real);
+  return sizeof(Real) == 8 ? (size_t)kBoysOrderLd * 8 : (size_t)Boys<Real>::NROW * Boys<Real>::NCOL * sizeof(Real);
 }
 
 template <typename Real>
@@ -328,7 +350,7 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
   constexpr bool kFlat = jk_flat<Real>();
   constexpr int L = LA + LB + LC + LD;
   constexpr int NFB = 4 + BC::NNZ;
-  constexpr int BK = Boys<Real>::NCOL, BR = Boys<Real>::NROW;
+  constexpr int BK = Boys<Real>::NCOL;
   constexpr int NWARP = kJKThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* sBoys = reinterpret_cast<Real*>(smem_raw);                     // [BR][BK]
@@ -338,8 +360,7 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
   Real* sJw = sDab + BC::NC;                    // per-bra form: per-warp J_bra partials [warp][a]
   Real* sbra = sJw + NWARP * BC::NC;            // per-bra form: bra primitive data [pp][field]
 
-  for (int x = threadIdx.x; x < BR * BK; x += blockDim.x)
-    sBoys[x] = P.boys[(x / BK) * kBoysCols + Boys<Real>::col(L, x % BK)];
+  stage_boys<Real, L>(sBoys, P.boys);
   __syncthreads();
   // thread = (chunk group cg, quartet q of the tile, bra-primitive subset bs);
   // the chunk group is the slowest index, so it is uniform within each warp

@@ -145,7 +145,8 @@ static long long screened_counts(const fsim_basis* b, int X, int Y, double tau, 
 
 // (Re)build the device work list of one class pair for a launch shape: on the
 // unrolled kernel psplit threads per quartet share the bra primitive pairs and
-// csplit thread groups share the ket chunks; or the cooperative kernel.
+// csplit thread groups share the ket chunks; or the cooperative kernel (flat:
+// the CTA-per-quartet kernel of generic.cuh, on the flattened quartet list).
 int set_class_plan(fsim_basis* b, int X, int Y, const std::vector<int>& count, int psplit, int coop,
                    ClassPairPlan& cp, int csplit, int flat) {
   const DevClass& CX = b->cls[X];
@@ -156,11 +157,11 @@ int set_class_plan(fsim_basis* b, int X, int Y, const std::vector<int>& count, i
   cp.coop = coop;
   cp.psplit = coop ? 1 : psplit;
   cp.csplit = coop ? 1 : csplit;
-  cp.tq = coop ? kCoopWarps : (kJKThreads / cp.csplit) / cp.psplit;
-  // tiles per bra (prefix of tile counts: cooperative kernel, per-bra form of
-  // the unrolled kernel) or tiles of the flattened (bra, ket) list (prefix of
-  // quartet counts: flattened form)
-  const bool fl = flat && !coop;
+  cp.tq = coop ? (flat ? 1 : kCoopWarps) : (kJKThreads / cp.csplit) / cp.psplit;
+  // tiles per bra (prefix of tile counts: warp-cooperative kernel, per-bra form
+  // of the unrolled kernel) or tiles of the flattened (bra, ket) list (prefix
+  // of quartet counts: flattened form; single quartets for a CTA each)
+  const bool fl = flat != 0;
   std::vector<int> prefix(CX.n + 1, 0);
   long long acc = 0;
   for (int i = 0; i < CX.n; ++i) {
@@ -185,6 +186,16 @@ int set_class_plan(fsim_basis* b, int X, int Y, const std::vector<int>& count, i
 static bool psplit_legal(const fsim_basis* b, int X, int Y, int ps) {
   if (ps == 27) return b->cls[X].ppmax >= 9 && b->cls[Y].ppmax >= 3;
   return (ps == 1 || ps == 3 || ps == 9) && ps <= b->cls[X].ppmax;
+}
+
+// Whether a build evaluates a class pair in FP64 with a CTA per quartet: the
+// heavy class pairs, and those with at most two waves of its CTAs, where the
+// unrolled kernel's threads, nine to a quartet, leave the FP64 pipes idle (six
+// (pp|pp) quartets: 35 against 201 us; 560 (pp|ps): 49 against 78; 1050
+// (pp|ss): 53 against 43).
+static bool plan_gen64(int precision, int X, int Y, long long nquartets) {
+  const bool in64 = precision == FSIM_FP64 || (precision == FSIM_DFLOAT && !dfloat_default(X, Y));
+  return in64 && (gen64_default(X, Y) || nquartets <= 6 * device_sm_count());
 }
 
 // Screened plan for (tau, shard, precision, psplit_force); cached on the basis.
@@ -212,7 +223,9 @@ int get_plan(fsim_basis* b, double tau, int shard, int nshards, int precision, F
       if (CX.n == 0 || b->cls[Y].n == 0) continue;
       std::vector<int> count;
       cp.nquartets = screened_counts(b, X, Y, tau, shard, nshards, count);
-      const int coop = 0;  // the cooperative kernel is an autotuner candidate only
+      // a batch's table (psplit_force > 0) holds tiles of the unrolled kernel
+      // only; the FP32 cooperative kernel is an autotuner candidate only
+      const int coop = psplit_force == 0 && plan_gen64(precision, X, Y, cp.nquartets);
       int ps = 1, cs = 1;
       {
         if (psplit_force > 0) {
@@ -252,41 +265,46 @@ int get_plan(fsim_basis* b, double tau, int shard, int nshards, int precision, F
   return FSIM_OK;
 }
 
-// The class pairs with an f class, on stream s (their quartet counts are below
-// 2^31 by set_class_plan's check).
+// One class pair with an f class on stream s (its quartet count is below 2^31 by
+// set_class_plan's check); a double-float build evaluates it in FP64.
+template <typename Real>
+static int launch_f_pair(fsim_basis* b, FockPlan* plan, int X, int Y, const Real* Dr, float boys64_T, double* Jacc,
+                         double* Kacc, cudaStream_t s, const double* D64) {
+  if constexpr (std::is_same<Real, dfloat>::value) {
+    return launch_f_pair<double>(b, plan, X, Y, D64, boys64_T, Jacc, Kacc, s, D64);
+  } else {
+    const ClassPairPlan& cp = plan->cp[X][Y];
+    if (cp.nquartets == 0) return FSIM_OK;
+    GenParams<Real> p{};
+    p.bra = b->cls[X].view<Real>();
+    p.ket = b->cls[Y].view<Real>();
+    p.la = pair_cls_la(X); p.lb = pair_cls_lb(X); p.lc = pair_cls_la(Y); p.ld = pair_cls_lb(Y);
+    p.same = X == Y;
+    p.list_mode = 0;
+    p.prefix = cp.d_prefix;
+    p.nitems = (int)cp.nquartets;
+    p.N = b->nbf;
+    p.D = Dr;
+    p.J = Jacc;
+    p.K = Kacc;
+    p.boys = std::is_same<Real, double>::value ? (const Real*)b->d_boys64 : (const Real*)b->d_boys32;
+    p.boys64_T = boys64_T;
+    const cudaError_t e = launch_gen<Real>(p, s);
+    ++b->last_launches;
+    if (e != cudaSuccess) {
+      set_error("J/K kernel for f class pair (%d|%d): %s", X, Y, cudaGetErrorString(e));
+      return FSIM_ECUDA;
+    }
+    return FSIM_OK;
+  }
+}
+
+// All class pairs with an f class, one after the other on stream s.
 template <typename Real>
 static int launch_f_pairs(fsim_basis* b, FockPlan* plan, const Real* Dr, float boys64_T, double* Jacc,
                           double* Kacc, cudaStream_t s, const double* D64 = nullptr) {
   for (int X = kNumPairClsAll - 1; X >= kNumPairCls; --X)
-    for (int Y = X; Y >= 0; --Y) {
-      const ClassPairPlan& cp = plan->cp[X][Y];
-      if (cp.nquartets == 0) continue;
-      cudaError_t e = cudaSuccess;
-      if constexpr (std::is_same<Real, dfloat>::value) {
-        return launch_f_pairs<double>(b, plan, D64, boys64_T, Jacc, Kacc, s);
-      } else {
-        GenParams<Real> p{};
-        p.bra = b->cls[X].view<Real>();
-        p.ket = b->cls[Y].view<Real>();
-        p.la = pair_cls_la(X); p.lb = pair_cls_lb(X); p.lc = pair_cls_la(Y); p.ld = pair_cls_lb(Y);
-        p.same = X == Y;
-        p.list_mode = 0;
-        p.prefix = cp.d_prefix;
-        p.nitems = (int)cp.nquartets;
-        p.N = b->nbf;
-        p.D = Dr;
-        p.J = Jacc;
-        p.K = Kacc;
-        p.boys = std::is_same<Real, double>::value ? (const Real*)b->d_boys64 : (const Real*)b->d_boys32;
-        p.boys64_T = boys64_T;
-        e = launch_gen<Real>(p, s);
-      }
-      ++b->last_launches;
-      if (e != cudaSuccess) {
-        set_error("J/K kernel for f class pair (%d|%d): %s", X, Y, cudaGetErrorString(e));
-        return FSIM_ECUDA;
-      }
-    }
+    for (int Y = X; Y >= 0; --Y) FSIM_TRY(launch_f_pair<Real>(b, plan, X, Y, Dr, boys64_T, Jacc, Kacc, s, D64));
   return FSIM_OK;
 }
 
@@ -327,11 +345,26 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
   if constexpr (std::is_same<Real, dfloat>::value) {
     if (!dfloat_kernel(X, Y) || cp.fp64) return launch_cp<double>(b, X, Y, cp, D64, Jacc, Kacc, boys64_T, s);
   }
-  const Real* boys = std::is_same<Real, double>::value   ? (const Real*)b->d_boys64
-                     : std::is_same<Real, float>::value  ? (const Real*)b->d_boys32
-                                                         : (const Real*)b->d_boysx;
   if (cp.nitems == 0) return cudaSuccess;
-  if constexpr (!std::is_same<Real, dfloat>::value) {  // the cooperative kernel exists in FP32 and FP64
+  if constexpr (std::is_same<Real, double>::value) {
+    if (cp.coop) {
+      GenParams<double> p{};
+      p.bra = b->cls[X].view<double>();
+      p.ket = b->cls[Y].view<double>();
+      p.la = pair_cls_la(X); p.lb = pair_cls_lb(X); p.lc = pair_cls_la(Y); p.ld = pair_cls_lb(Y);
+      p.same = X == Y ? 1 : 0;
+      p.prefix = cp.d_prefix;
+      p.nitems = cp.nitems;
+      p.N = b->nbf;
+      p.D = Dr;
+      p.J = Jacc;
+      p.K = Kacc;
+      p.boys = b->d_boys64;
+      p.boys64_T = boys64_T;
+      return launch_gen<double>(p, s);
+    }
+  }
+  if constexpr (std::is_same<Real, float>::value) {
     if (cp.coop) {
       CoopParams<Real> p{};
       p.bra = b->cls[X].view<Real>();
@@ -348,7 +381,7 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
       p.D = Dr;
       p.J = Jacc;
       p.K = Kacc;
-      p.boys = boys;
+      p.boys = b->d_boys32;
       p.boys64_T = boys64_T;
       return launch_coop<Real>(p, cp.nitems, s);
     }
@@ -360,7 +393,7 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
   p.psplit = cp.psplit;
   p.csplit = cp.csplit;
   p.bra_ppmax = b->cls[X].ppmax;
-  p.boys = boys;
+  p.boys = quartet_boys<Real>(b);
   p.boys64_T = boys64_T;
   return dispatch_jk<Real>(X, Y, p, s);
 }
@@ -410,6 +443,10 @@ static int launch_all(fsim_basis* b, FockPlan* plan, const Real* Dr, float boys6
         b->last_class_run[ci] = cp.nitems > 0;
         if (cp.nitems > 0) jobs.push_back(Job{X, Y, (double)cp.nquartets * class_cost(X, Y)});
       }
+    for (int X = kNumPairClsAll - 1; X >= kNumPairCls; --X)
+      for (int Y = X; Y >= 0; --Y)
+        if (plan->cp[X][Y].nquartets > 0)
+          jobs.push_back(Job{X, Y, (double)plan->cp[X][Y].nquartets * class_cost(X, Y)});
     std::stable_sort(jobs.begin(), jobs.end(), [](const Job& a, const Job& c) { return a.cost > c.cost; });
     constexpr int NS = fsim_basis::kAuxStreams + 1;
     cudaStream_t st[NS] = {s};
@@ -423,6 +460,10 @@ static int launch_all(fsim_basis* b, FockPlan* plan, const Real* Dr, float boys6
       for (int t = 1; t < nuse; ++t)
         if (load[t] < load[k]) k = t;
       load[k] += j.cost;
+      if (j.X >= kNumPairCls) {
+        FSIM_TRY(launch_f_pair<Real>(b, plan, j.X, j.Y, Dr, boys64_T, b->d_Jacc, b->d_Kacc, st[k], D64));
+        continue;
+      }
       ++b->last_launches;
       const cudaError_t e = launch_cp<Real>(b, j.X, j.Y, plan->cp[j.X][j.Y], Dr, b->d_Jacc, b->d_Kacc, boys64_T,
                                             st[k], D64);
@@ -431,7 +472,6 @@ static int launch_all(fsim_basis* b, FockPlan* plan, const Real* Dr, float boys6
         return FSIM_ECUDA;
       }
     }
-    FSIM_TRY(launch_f_pairs<Real>(b, plan, Dr, boys64_T, b->d_Jacc, b->d_Kacc, s, D64));
     for (int k = 1; k < nuse; ++k) {
       FSIM_CK(cudaEventRecord(b->join_ev[k - 1], st[k]));
       FSIM_CK(cudaStreamWaitEvent(s, b->join_ev[k - 1], 0));
@@ -842,7 +882,10 @@ static int autotune_impl(fsim_basis* b, FockPlan* plan, const Real* Dr, float b6
           for (int cs : {1, 2, 4})
             if (psplit_legal(b, X, Y, ps) && cs <= nch && (ps < 27 || cp.nquartets * 9 < fill))
               cands.push_back({ps, 0, cs, f64});
+      // the cooperative kernel; a double-float build has it where it is the
+      // class pair's default (reported as 0, fsim_set_launch's "as planned")
       if (!kDf) cands.push_back({1, 1, 1, 0});
+      else if (plan_gen64(FSIM_DFLOAT, X, Y, cp.nquartets)) cands.push_back({1, 1, 1, 1});
       float best = 1e30f;
       Cand win = cands[0];
       ClassPairPlan tmp;
@@ -875,7 +918,7 @@ static int autotune_impl(fsim_basis* b, FockPlan* plan, const Real* Dr, float b6
       if (rc != FSIM_OK) break;
       rc = set_class_plan(b, X, Y, count, win.psplit, win.coop, cp, win.csplit, jk_flat<Real>());
       cp.fp64 = win.fp64;
-      if (choice) choice[ci] = win.coop ? -1 : 10 * win.psplit + win.csplit + 1000 * win.fp64;
+      if (choice) choice[ci] = win.coop ? (kDf ? 0 : -1) : 10 * win.psplit + win.csplit + 1000 * win.fp64;
       if (best_ms) best_ms[ci] = best;
     }
   cudaEventDestroy(e0);

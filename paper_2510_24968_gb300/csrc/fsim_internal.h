@@ -159,6 +159,13 @@ __host__ __device__ constexpr bool dfloat_kernel(int X, int Y) { return !(X == 5
 __host__ __device__ constexpr bool dfloat_default(int X, int Y) {
   return dfloat_kernel(X, Y) && pair_cls_la(X) + pair_cls_lb(X) + pair_cls_la(Y) + pair_cls_lb(Y) <= 4;
 }
+// Class pairs whose FP64 evaluation takes the CTA-per-quartet kernel
+// (generic.cuh) instead of the unrolled one: where the ket transform, H(bra) x
+// non-zeros(ket) multiply-adds per primitive quartet, outweighs what the former
+// spends per primitive quartet at 27 of 32 lanes.
+__host__ __device__ constexpr bool gen64_default(int X, int Y) {
+  return nherm(pair_cls_la(X) + pair_cls_lb(X)) * pair_cls_nnz(Y) >= 600;
+}
 static_assert(sizeof(dfloat) == sizeof(double), "double-float values share the FP64 layouts and chunk sizes");
 
 // Ket chunks of the unrolled kernel for a class pair (host side of KetChunks).
@@ -174,7 +181,7 @@ struct ClassPairPlan {
   long long nquartets = 0;
   int psplit = 1;
   int csplit = 1;           // ket chunk groups per CTA (unrolled kernel)
-  int coop = 0;             // 1: warp-cooperative table-driven kernel
+  int coop = 0;             // 1: table-driven kernel, a warp (FP32) or a CTA (FP64) per quartet
   int fp64 = 0;             // FSIM_DFLOAT plans: 1 = this class pair runs the FP64 kernel
   int tq = kJKThreads;      // kets per work item
   int* d_prefix = nullptr;  // [nbra + 1]
@@ -250,9 +257,10 @@ struct fsim_basis {
   fsim::DevClass cls[fsim::kNumPairClsAll];
   bool schwarz_done = false;
   std::vector<double> Q;  // nshell x nshell
-  double* d_boys64 = nullptr;
+  double* d_boys64 = nullptr;       // full tables, rows of kBoysCols
   float* d_boys32 = nullptr;
-  fsim::dfloat* d_boysx = nullptr;  // double-float copy of the FP64 table (first FSIM_DFLOAT use)
+  double* d_boys64s = nullptr;      // per class order, as the quartet kernels stage them (boys.cuh)
+  fsim::dfloat* d_boysx = nullptr;  // the same in double-float (first FSIM_DFLOAT use)
   bool dfloat_ready = false;
   std::vector<fsim::FockPlan*> plans;
   std::vector<fsim::JPlan*> jplans;
@@ -284,6 +292,13 @@ struct fsim_basis {
 };
 
 namespace fsim {
+// the Boys table the quartet kernels of a precision stage (stage_boys)
+template <typename Real>
+inline const Real* quartet_boys(const fsim_basis* b) {
+  if constexpr (std::is_same<Real, double>::value) return b->d_boys64s;
+  else if constexpr (std::is_same<Real, float>::value) return b->d_boys32;
+  else return b->d_boysx;
+}
 int get_plan(fsim_basis* b, double tau, int shard, int nshards, int precision, FockPlan** out, int psplit_force);
 int set_class_plan(fsim_basis* b, int X, int Y, const std::vector<int>& count, int psplit, int coop,
                    ClassPairPlan& cp, int csplit, int flat);

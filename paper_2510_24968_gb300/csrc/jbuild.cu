@@ -174,7 +174,7 @@ static int jeng_launch_all(fsim_basis* b, JPlan* plan, const Real* Dr, float b64
   FSIM_CK(cudaEventRecord(b->fork_ev, s));
   for (int k = 1; k < nuse; ++k) FSIM_CK(cudaStreamWaitEvent(st[k], b->fork_ev, 0));
   double load[NS] = {};
-  const Real* boys = std::is_same<Real, double>::value ? (const Real*)b->d_boys64 : (const Real*)b->d_boys32;
+  const Real* boys = quartet_boys<Real>(b);
   for (const Job& jb : jobs) {
     int k = 0;
     for (int t = 1; t < nuse; ++t)

@@ -89,15 +89,14 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
   constexpr int L = LA + LB + LC + LD;
   constexpr int NH = nherm(L), NH1 = BC::NH, NH2 = KC::NH;
   constexpr int NFB = 4 + BC::NNZ;
-  constexpr int BK = Boys<Real>::NCOL, BR = Boys<Real>::NROW;
+  constexpr int BK = Boys<Real>::NCOL;
   constexpr int NWARP = kJKThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* sBoys = reinterpret_cast<Real*>(smem_raw);
   Real* sJ = reinterpret_cast<Real*>(smem_raw + (jk_boys_smem<Real>() + 15) / 16 * 16);  // [a][thread]
   Real* sJw = sJ + BC::NC * kJKThreads;                                                    // [warp][a]
   Real* sbra = sJw + NWARP * BC::NC;                                                       // [pp][field]
-  for (int x = threadIdx.x; x < BR * BK; x += blockDim.x)
-    sBoys[x] = P.boys[(x / BK) * kBoysCols + Boys<Real>::col(L, x % BK)];
+  stage_boys<Real, L>(sBoys, P.boys);
   const int ps = P.psplit, tq = kJKThreads / ps;
   const int q = threadIdx.x / ps, bs = threadIdx.x % ps;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -127,21 +126,9 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
         for (int k = 0; k < nppk; ++k) {
           const auto q4 = P.ket.pq[(size_t)k * P.ket.n + j];
           const Real qq = q4.x;
-          const Real s = p + qq;
-          const Real rs = rsqrt_r<Real>(s);
-          const Real al = p * qq * (rs * rs);
           const Real X = Px - q4.y, Y = Py - q4.z, Z = Pz - q4.w;
-          const Real T = al * (X * X + Y * Y + Z * Z);
-          Real F[L + 1];
-          Boys<Real>::template eval<L>(T, F, sBoys, BK, P.boys64_T);
           Real src[L + 1];
-          Real fac = rs;
-          const Real m2a = Real(-2) * al;
-#pragma unroll
-          for (int n = 0; n <= L; ++n) {
-            src[n] = fac * F[n];
-            fac *= m2a;
-          }
+          prim_sources<Real, L>(p, qq, X, Y, Z, src, sBoys, BK, P.boys64_T);
           Real R[NH];
           hermite_R<Real, L>(R, src, X, Y, Z);
           const Real* rk = P.rho + (size_t)k * P.ket.n + j;
