@@ -127,7 +127,8 @@ struct fsim_batch {
   double tau = 0.0;
   cudaStream_t s = nullptr;
   struct CPB {
-    int nitems = 0, bra_ppmax = 1, nin = 0;
+    int nitems = 0, bra_ppmax = 1, nin = 0, psplit = 1;
+    double cost = 0.0;
     void* d_mols = nullptr;
     int* d_prefix = nullptr;
     int* d_ids = nullptr;
@@ -140,6 +141,10 @@ struct fsim_batch {
   fsim::MolPtrs* d_ptrs = nullptr;
   std::vector<fsim::MolPtrs> h_ptrs;
   int maxN = 0;
+  // the class-pair launches of a build run side by side on these and bt->s
+  static constexpr int kAux = 3;
+  cudaStream_t aux[kAux] = {};
+  cudaEvent_t fork_ev = nullptr, join_ev[kAux] = {};
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
   cudaGraph_t graph[2] = {nullptr, nullptr};
 };
@@ -155,10 +160,26 @@ int build_tables(fsim_batch* bt, int prec) {
       std::vector<JKMol<Real>> mols;
       std::vector<int> prefix(1, 0);
       C.ids.clear();
+      // FP64: class pairs with fewer quartets in the whole batch than two CTAs
+      // per SM have threads give each quartet nine threads, one per bra primitive
+      // pair.  (FP32 sums J_bra over 32 kets in FP32; other tiles would change
+      // its rounding.)
+      long long nq = 0;
+      bool nine = true;
+      for (int m = 0; m < bt->nmol; ++m) {
+        FockPlan* plan = nullptr;
+        FSIM_TRY(get_plan(bt->b[m], bt->tau, 0, 1, prec == 0 ? FSIM_FP64 : FSIM_MIXED, &plan, 1));
+        nq += plan->cp[X][Y].nquartets;
+        if (plan->cp[X][Y].nquartets > 0 && bt->b[m]->cls[X].ppmax < 9) nine = false;
+      }
+      const long long fill = (long long)device_sm_count() * 2 * kJKThreads;
+      C.psplit = nine && prec == 0 && nq < fill ? 9 : 1;
+      // a launch that does not fill the device takes as long as one that does
+      C.cost = (double)std::max(nq, fill / C.psplit) * class_cost(X, Y);
       for (int m = 0; m < bt->nmol; ++m) {
         fsim_basis* b = bt->b[m];
         FockPlan* plan = nullptr;
-        FSIM_TRY(get_plan(b, bt->tau, 0, 1, prec == 0 ? FSIM_FP64 : FSIM_MIXED, &plan, 1));
+        FSIM_TRY(get_plan(b, bt->tau, 0, 1, prec == 0 ? FSIM_FP64 : FSIM_MIXED, &plan, C.psplit));
         const ClassPairPlan& cp = plan->cp[X][Y];
         if (cp.nitems == 0) continue;
         const Real* D = prec == 0 ? (const Real*)bt->h_ptrs[m].Din : (const Real*)bt->h_ptrs[m].D32;
@@ -197,34 +218,61 @@ int launch_batch(fsim_batch* bt, int prec, cudaStream_t s, bool dry) {
     batch_prepare_kernel<<<g, 256, 0, s>>>(bt->d_ptrs, bt->d_active, mixed);
     FSIM_CK(cudaGetLastError());
   }
-  for (int X = kNumPairCls - 1; X >= 0; --X)
-    for (int Y = X; Y >= 0; --Y) {
-      const fsim_batch::CPB& C = bt->cp[prec][X][Y];
-      if (C.nin == 0) continue;
-      cudaError_t e = cudaSuccess;
-      {
-        JKParams<Real> p{};
-        p.mols = (const JKMol<Real>*)C.d_mols;
-        p.mol_prefix = C.d_prefix;
-        p.active = bt->d_active;
-        p.tau_mol = bt->d_tau;
-        p.mol_ids = C.d_ids;
-        p.nmol = C.nin;
-        p.nitems = dry ? 0 : C.nitems;
-        p.same = X == Y ? 1 : 0;
-        p.psplit = 1;
-        p.csplit = 1;
-        p.bra_ppmax = C.bra_ppmax;
-        p.boys = quartet_boys<Real>(bt->b[0]);
-        p.boys64_T = INFINITY;
-        e = dispatch<Real>(X, Y, p, s);
-      }
-      if (e != cudaSuccess) {
-        set_error("batched J/K (%d|%d): %s", X, Y, cudaGetErrorString(e));
-        return FSIM_ECUDA;
-      }
+  // longest first onto the least loaded stream, between a fork and a join
+  // event: most launches of a batch of small molecules leave part of the device
+  // idle (in one chain, 24 clusters (H2O)_2..6 took the sum of 21 latencies)
+  std::vector<std::pair<int, int>> order;
+  for (int X = 0; X < kNumPairCls; ++X)
+    for (int Y = 0; Y <= X; ++Y)
+      if (bt->cp[prec][X][Y].nin > 0) order.push_back({X, Y});
+  std::stable_sort(order.begin(), order.end(), [&](const std::pair<int, int>& a, const std::pair<int, int>& c) {
+    return bt->cp[prec][a.first][a.second].cost > bt->cp[prec][c.first][c.second].cost;
+  });
+  constexpr int NS = fsim_batch::kAux + 1;
+  cudaStream_t st[NS] = {s};
+  for (int k = 0; k < fsim_batch::kAux; ++k) st[k + 1] = bt->aux[k];
+  double load[NS] = {};
+  if (!dry) {
+    FSIM_CK(cudaEventRecord(bt->fork_ev, s));
+    for (int k = 1; k < NS; ++k) FSIM_CK(cudaStreamWaitEvent(st[k], bt->fork_ev, 0));
+  }
+  int rc = FSIM_OK;
+  for (const auto& [X, Y] : order) {
+    const fsim_batch::CPB& C = bt->cp[prec][X][Y];
+    int k = 0;
+    for (int t = 1; t < NS; ++t)
+      if (load[t] < load[k]) k = t;
+    load[k] += C.cost;
+    cudaError_t e = cudaSuccess;
+    {
+      JKParams<Real> p{};
+      p.mols = (const JKMol<Real>*)C.d_mols;
+      p.mol_prefix = C.d_prefix;
+      p.active = bt->d_active;
+      p.tau_mol = bt->d_tau;
+      p.mol_ids = C.d_ids;
+      p.nmol = C.nin;
+      p.nitems = dry ? 0 : C.nitems;
+      p.same = X == Y ? 1 : 0;
+      p.psplit = C.psplit;
+      p.csplit = 1;
+      p.bra_ppmax = C.bra_ppmax;
+      p.boys = quartet_boys<Real>(bt->b[0]);
+      p.boys64_T = INFINITY;
+      e = dispatch<Real>(X, Y, p, st[k]);
     }
-  if (dry) return FSIM_OK;
+    if (e != cudaSuccess) {
+      set_error("batched J/K (%d|%d): %s", X, Y, cudaGetErrorString(e));
+      rc = FSIM_ECUDA;
+      break;
+    }
+  }
+  if (dry) return rc;
+  for (int k = 1; k < NS; ++k) {  // after an error too: no stream is left unjoined
+    FSIM_CK(cudaEventRecord(bt->join_ev[k - 1], st[k]));
+    FSIM_CK(cudaStreamWaitEvent(s, bt->join_ev[k - 1], 0));
+  }
+  if (rc != FSIM_OK) return rc;
   dim3 g2(std::max(1, std::min(64, (bt->maxN * bt->maxN + 255) / 256)), bt->nmol);
   batch_symmetrize_kernel<<<g2, 256, 0, s>>>(bt->d_ptrs, bt->d_active);
   FSIM_CK(cudaGetLastError());
@@ -288,6 +336,16 @@ int fsim_batch_create(fsim_basis* const* bases, int nmol, const fsim_fock_opts* 
     set_error("fsim_batch_create: upload failed");
     return fail(FSIM_ECUDA);
   }
+  for (int k = 0; k < fsim_batch::kAux; ++k)
+    if (cudaStreamCreateWithFlags(&bt->aux[k], cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&bt->join_ev[k], cudaEventDisableTiming) != cudaSuccess) {
+      set_error("fsim_batch_create: stream or event creation failed");
+      return fail(FSIM_ECUDA);
+    }
+  if (cudaEventCreateWithFlags(&bt->fork_ev, cudaEventDisableTiming) != cudaSuccess) {
+    set_error("fsim_batch_create: event creation failed");
+    return fail(FSIM_ECUDA);
+  }
   if ((rc = build_tables<double>(bt, 0)) != FSIM_OK || (rc = build_tables<float>(bt, 1)) != FSIM_OK) return fail(rc);
   *out = bt;
   return FSIM_OK;
@@ -305,6 +363,11 @@ void fsim_batch_destroy(fsim_batch* bt) {
         dev_free(C.d_ids);
       }
   }
+  for (int k = 0; k < fsim_batch::kAux; ++k) {
+    if (bt->aux[k]) cudaStreamDestroy(bt->aux[k]);
+    if (bt->join_ev[k]) cudaEventDestroy(bt->join_ev[k]);
+  }
+  if (bt->fork_ev) cudaEventDestroy(bt->fork_ev);
   dev_free(bt->d_active);
   dev_free(bt->d_tau);
   dev_free(bt->d_incr);

@@ -400,7 +400,7 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
 
 // Relative cost of one quartet of a class pair: the algorithmic flop count per
 // primitive quartet (R recursion + the cheaper contraction order).
-static double class_cost(int X, int Y) {
+double class_cost(int X, int Y) {
   const int la = pair_cls_la(X), lb = pair_cls_lb(X), lc = pair_cls_la(Y), ld = pair_cls_lb(Y);
   const double A = ncart(la) * ncart(lb), C = ncart(lc) * ncart(ld);
   const double H1 = nherm(la + lb), H2 = nherm(lc + ld);

@@ -326,6 +326,7 @@ inline bool has_f(const fsim_basis* b);
 // input, hidden and output widths of a network handle (mlp.cu)
 void mlp_dims(const fsim_mlp* net, int* nin, int* width, int* nout);
 int device_sm_count();
+double class_cost(int X, int Y);
 int build_pair_data(fsim_basis* b, int cls, const std::vector<int4>& order);
 int run_list(fsim_basis* b, int X, int Y, const std::vector<int2>& items, double* d_out, int precision,
              cudaStream_t s);
