@@ -101,6 +101,53 @@ int build_pair_data(fsim_basis* b, int cls, const std::vector<int4>& order) {
   return FSIM_OK;
 }
 
+// Bounds of the primitive pairs (prim_mask's bytes): for one primitive pair, T = 0
+// and (ab_a|ab_a) = sum_{h,h'} E_h E_h' (-1)^{|h'|} R_{h+h'} with R_{tuv} zero for an
+// odd index and (t-1)!!(u-1)!!(v-1)!! (-p)^n / ((2n+1) sqrt(2p)), n = (t+u+v)/2,
+// otherwise.  One thread per pair and primitive pair; runtime loops, FP64.
+__global__ void prim_bound_kernel(int n, int ppmax, int la, int lb, const int* __restrict__ npp,
+                                  const double* __restrict__ pd, unsigned char* __restrict__ ub) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = x % n, k = x / n;
+  if (k >= 16) return;
+  unsigned char byte = 0x80;  // padding: below every threshold
+  if (k < npp[j]) {
+    const size_t fs = (size_t)ppmax * n;
+    const double* e = pd + (size_t)k * n + j;
+    const double p = e[0];
+    constexpr double odd[7] = {1, 1, 3, 15, 105, 945, 10395};  // (2m - 1)!!
+    double best = 0.0;
+    int z0 = 4;
+    for (int a = 0; a < ncart(la) * ncart(lb); ++a) {
+      int ext[3];
+      for (int d = 0; d < 3; ++d) ext[d] = cart_comp(la, a / ncart(lb), d) + cart_comp(lb, a % ncart(lb), d);
+      const int su = ext[2] + 1, st = (ext[1] + 1) * su, nz = (ext[0] + 1) * st;
+      double v = 0.0;
+      for (int h = 0; h < nz; ++h) {
+        const int t = h / st, u = h / su % (ext[1] + 1), w = h % su;
+        double row = 0.0;
+        for (int t2 = t & 1; t2 <= ext[0]; t2 += 2)
+          for (int u2 = u & 1; u2 <= ext[1]; u2 += 2)
+            for (int w2 = w & 1; w2 <= ext[2]; w2 += 2) {
+              const int m = (t + t2 + u + u2 + w + w2) / 2;
+              double r = odd[(t + t2) / 2] * odd[(u + u2) / 2] * odd[(w + w2) / 2] / (2 * m + 1);
+              for (int i = 0; i < m; ++i) r *= -p;
+              if ((t2 + u2 + w2) & 1) r = -r;
+              row = fma(e[(size_t)(z0 + t2 * st + u2 * su + w2) * fs], r, row);
+            }
+        v = fma(e[(size_t)(z0 + h) * fs], row, v);
+      }
+      z0 += nz;
+      best = v == v ? fmax(best, fabs(v)) : INFINITY;  // (an earlier infinity stays)
+    }
+    int ex = 0;
+    frexp(sqrt(best / sqrt(2.0 * p)) * (1.0 + 1e-9), &ex);  // q < 2^ex
+    const int c = best > 0.0 ? ex + kPrimBias : 0;
+    byte = (unsigned char)(0x80 | (c < 0 ? 0 : (c >= kPrimNoBound || !(best < 1e300) ? kPrimNoBound : c)));
+  }
+  ub[16 * (size_t)j + k] = byte;
+}
+
 // Double-float copies (nearest dfloat of each FP64 value) of the pair data, the
 // Boys table and a density buffer, made once on the first FSIM_DFLOAT build.
 __global__ void split_kernel(const double* __restrict__ in, dfloat* __restrict__ out, size_t n) {
@@ -308,6 +355,11 @@ static int compute_schwarz(fsim_basis* b) {
       C.h_Q[j] = q[perm[j]];
     }
     FSIM_TRY(build_pair_data(b, X, order));
+    dev_free(C.ub);
+    FSIM_TRY(dev_alloc(&C.ub, C.n));
+    prim_bound_kernel<<<(C.n * 16 + 127) / 128, 128>>>(C.n, C.ppmax, pair_cls_la(X), pair_cls_lb(X), C.npp, C.pd64,
+                                                       reinterpret_cast<unsigned char*>(C.ub));
+    FSIM_CK(cudaGetLastError());
     if (!C.d_Q) FSIM_TRY(dev_alloc(&C.d_Q, std::max(C.n, 1)));
     if (C.n) FSIM_CK(cudaMemcpy(C.d_Q, C.h_Q.data(), sizeof(double) * C.n, cudaMemcpyHostToDevice));
   }
@@ -455,7 +507,7 @@ void fsim_basis_destroy(fsim_basis* b) {
   if (!b) return;
   for (auto& C : b->cls) {
     dev_free(C.idx); dev_free(C.npp); dev_free(C.pd64); dev_free(C.pd32); dev_free(C.pq64); dev_free(C.pq32);
-    dev_free(C.pdx); dev_free(C.pqx); dev_free(C.d_Q);
+    dev_free(C.pdx); dev_free(C.pqx); dev_free(C.d_Q); dev_free(C.ub);
   }
   for (auto* p : b->plans) {
     for (auto& row : p->cp)

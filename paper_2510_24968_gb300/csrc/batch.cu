@@ -128,6 +128,7 @@ struct fsim_batch {
   cudaStream_t s = nullptr;
   struct CPB {
     int nitems = 0, bra_ppmax = 1, nin = 0, psplit = 1;
+    int prim_lt = fsim::kPrimKeepAll;
     double cost = 0.0;
     void* d_mols = nullptr;
     int* d_prefix = nullptr;
@@ -174,6 +175,7 @@ int build_tables(fsim_batch* bt, int prec) {
       }
       const long long fill = (long long)device_sm_count() * 2 * kJKThreads;
       C.psplit = nine && prec == 0 && nq < fill ? 9 : 1;
+      C.prim_lt = prim_threshold(bt->tau, prec == 1);
       // a launch that does not fill the device takes as long as one that does
       C.cost = (double)std::max(nq, fill / C.psplit) * class_cost(X, Y);
       for (int m = 0; m < bt->nmol; ++m) {
@@ -220,7 +222,7 @@ int launch_batch(fsim_batch* bt, int prec, cudaStream_t s, bool dry) {
   }
   // longest first onto the least loaded stream, between a fork and a join
   // event: most launches of a batch of small molecules leave part of the device
-  // idle (in one chain, 24 clusters (H2O)_2..6 took the sum of 21 latencies)
+  // idle (24 clusters (H2O)_2..6, mixed: one chain 5.7 ms, four streams 3.4)
   std::vector<std::pair<int, int>> order;
   for (int X = 0; X < kNumPairCls; ++X)
     for (int Y = 0; Y <= X; ++Y)
@@ -255,6 +257,7 @@ int launch_batch(fsim_batch* bt, int prec, cudaStream_t s, bool dry) {
       p.nitems = dry ? 0 : C.nitems;
       p.same = X == Y ? 1 : 0;
       p.psplit = C.psplit;
+      p.prim_lt = C.prim_lt;
       p.csplit = 1;
       p.bra_ppmax = C.bra_ppmax;
       p.boys = quartet_boys<Real>(bt->b[0]);

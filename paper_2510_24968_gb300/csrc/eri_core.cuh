@@ -54,7 +54,56 @@ struct PairView {
   const int* __restrict__ npp;                      // primitive pairs of each pair
   const Real* __restrict__ pd;                      // [field][pp][pair]
   const typename Vec4<Real>::type* __restrict__ pq;  // (p, Px, Py, Pz) at [pp][pair]
+  const uint4* __restrict__ ub;                      // Schwarz bounds of the pair's primitive pairs (prim_mask)
 };
+
+// Primitive quartets that cannot matter.  |(ab|cd)| of a primitive quartet is at
+// most q_ab q_cd, q_ab = sqrt(max_a |(ab_a|ab_a)|) of one primitive pair (Schwarz),
+// and the bounds of one contracted pair of distant centres span many orders of
+// magnitude.  A primitive quartet whose bound is below a threshold theta is left
+// out of the contraction: theta is a power of two at most 2^-20 of the screening
+// threshold and 2^-53 (FP64, double-float), or 2^-13 of it and 2^-43 (FP32), so
+// that all that is left out stays below the rounding of the integrals themselves
+// (prim_threshold; nothing is left out at screening threshold 0).  (H2O)_8 at
+// 1e-10 needs 60-70 % of its primitive quartets at the FP64 threshold (61.7 ->
+// 48.5 ms), the compact 7-atom cloud nearly all of them (55.4 ms both ways).
+//
+// Per pair, one byte per primitive pair: 0x80 | clamp(e + 96, 0, 127) with
+// q < 2^e; 127 means "no bound".
+constexpr int kPrimBias = 96, kPrimNoBound = 127;
+constexpr int kPrimKeepAll = -100000;  // log2 theta of an unscreened build
+
+// Kernels of order L that skip: FP64 (bound by its arithmetic) all of them; FP32
+// and double-float those whose unrolled bodies are short.  The others are bound
+// by instruction supply, which their warps share while they run in step, and
+// skipping puts them out of step (30-atom cloud, FP32: (dp|ps) 46 -> 38 ms, but
+// (dd|dp) 60 -> 77; 12-atom cloud: (dp|pp) 2.14 -> 2.26; (H2O)_8, double-float:
+// (ps|ss) 1.47 -> 1.08 ms, but (dp|ps) 1.9 -> 4.3).
+template <typename Real>
+__host__ __device__ constexpr bool prim_skip(int L) {
+  return std::is_same<Real, double>::value || (std::is_same<Real, float>::value ? L <= 4 : L <= 2);
+}
+
+// byte of primitive pair b
+__device__ __forceinline__ int prim_byte(const uint4* ub, int b) {
+  return __ldg(reinterpret_cast<const unsigned char*>(ub) + b) & 0x7f;
+}
+// smallest byte of the other side that is kept beside byte vb; log2_theta: theta = 2^log2_theta
+__host__ __device__ __forceinline__ int prim_least(int log2_theta, int vb) {
+  const int t = log2_theta + 1 - (vb - kPrimBias) + kPrimBias;
+  return vb == kPrimNoBound || t < 0 ? 0 : (t > 127 ? 127 : t);
+}
+// bit k set: primitive pair k < npp <= 16 is kept; bytes compared four at a time
+// (the guard bit of a byte survives the subtraction where it is at least `least`)
+__host__ __device__ __forceinline__ unsigned prim_mask(uint4 v, int least, int npp) {
+  const unsigned t = 0x01010101u * (unsigned)least;
+  auto four = [&](unsigned w) { return ((((w - t) >> 7) & 0x01010101u) * 0x10204080u) >> 28; };
+  unsigned m = four(v.x);
+  if (npp > 4) m |= four(v.y) << 4;
+  if (npp > 8) m |= four(v.z) << 8;
+  if (npp > 12) m |= four(v.w) << 12;
+  return m & ((1u << npp) - 1u);
+}
 
 // Everything a work item needs about its molecule.
 template <typename Real>
@@ -87,6 +136,7 @@ struct JKParams {
   int bra_ppmax;                        // largest bra primitive-pair count (shared-memory size)
   const Real* __restrict__ boys;
   float boys64_T;                       // FP32 path: Boys in FP64 at T >= this (infinity = never)
+  int prim_lt;                          // log2 of the primitive-quartet threshold (prim_mask)
   // batched, optional: per molecule (indexed like active) a density-weighted
   // threshold; a quartet with Q_ab Q_cd below it is skipped (0: none skipped)
   const float* __restrict__ tau_mol = nullptr;
@@ -192,6 +242,8 @@ struct KetChunks {
 // a and ket components c = ch*CS + cs < NC, accumulated in this thread's
 // shared-memory slots so[(a * CS + cs) * kJKThreads] (so the registers hold
 // only R, the chunk's W and its E non-zeros).  Bra data: accessor bra(field, pp).
+// Primitive quartets below the threshold 2^prim_lt are skipped (prim_mask; bub:
+// the bra's bounds).
 // The bstep threads of a quartet share its primitive quartets: with bstep <=
 // nppb each takes whole bra primitive pairs (b0, b0 + bstep, ...) and every ket
 // primitive pair; with more threads than bra primitive pairs the ket primitive
@@ -206,8 +258,9 @@ struct KetChunks {
 // the instruction footprint of a chunk small enough for the instruction cache.
 template <typename Real, int LA, int LB, int LC, int LD, int CS, class BraAt>
 __device__ __forceinline__ void quartet_chunk(Real* __restrict__ so, const BraAt& bra, int nppb, int b0, int bstep,
-                                              const PairView<Real>& ket, int j, int nppk,
-                                              const Real* __restrict__ boysL, int bstride, float t64, int ch) {
+                                              const PairView<Real>& ket, int j, int nppk, const uint4* bub, int prim_lt,
+                                              const Real* __restrict__ boysL, int bstride, float t64,
+                                              int ch) {
   using BC = PairCls<LA, LB>;
   using KC = PairCls<LC, LD>;
   using KCh = KetChunks<KC, CS>;
@@ -215,19 +268,31 @@ __device__ __forceinline__ void quartet_chunk(Real* __restrict__ so, const BraAt
   constexpr int NH = nherm(L);
   constexpr int NH1 = BC::NH;
   constexpr int NZM = KCh::max_nnz();
+  constexpr bool kSkip = prim_skip<Real>(L);
 #pragma unroll
   for (int x = 0; x < BC::NC * CS; ++x) so[x * kJKThreads] = Real(0);
   const size_t kstride = (size_t)ket.ppmax * ket.n;
   const int ks = (bstep + nppb - 1) / nppb;
   for (int u = b0; u < nppb * ks; u += bstep) {
     const int b = u % nppb;
+    // the ket primitive pairs to take with this bra primitive pair: every ks-th from u / nppb
+    unsigned todo = 0;
+    if constexpr (kSkip) {
+      todo = prim_mask(__ldg(ket.ub + j), prim_least(prim_lt, prim_byte(bub, b)), nppk);
+      if (ks > 1)
+        for (int k = 0; k < nppk; ++k)
+          if (k % ks != u / nppb) todo &= ~(1u << k);
+      if (todo == 0) continue;
+    }
     const Real p = bra(0, b), Px = bra(1, b), Py = bra(2, b), Pz = bra(3, b);
     Real W[NH1][CS];
 #pragma unroll
     for (int h = 0; h < NH1; ++h)
 #pragma unroll
       for (int cs = 0; cs < CS; ++cs) W[h][cs] = Real(0);
-    for (int k = u / nppb; k < nppk; k += ks) {
+    for (int k = kSkip ? __ffs(todo) - 1 : u / nppb; kSkip ? todo != 0 : k < nppk;
+         k = kSkip ? __ffs(todo) - 1 : k + ks) {
+      todo &= todo - 1;
       const Real* kp = ket.pd + (size_t)k * ket.n + j;
       const auto q4 = ket.pq[(size_t)k * ket.n + j];
       const Real q = q4.x, Qx = q4.y, Qy = q4.z, Qz = q4.w;
@@ -442,7 +507,8 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
 #pragma unroll 1
       for (int ch = cg; ch < KetChunks<KC, CS>::NCH; ch += ncg) {
         if (valid)
-          quartet_chunk<Real, LA, LB, LC, LD, CS>(so, bra, nppb, bs, ps, M.ket, j, nppk, sBoys, BK, P.boys64_T, ch);
+          quartet_chunk<Real, LA, LB, LC, LD, CS>(so, bra, nppb, bs, ps, M.ket, j, nppk, M.bra.ub + i, P.prim_lt,
+                                                  sBoys, BK, P.boys64_T, ch);
         if (ps > 1) {
           // the ps threads of a quartet hold partial blocks over their bra
           // primitive pairs: sum them into the first thread's slots (each

@@ -90,6 +90,7 @@ int run_list(fsim_basis* b, int X, int Y, const std::vector<int2>& items, double
     p.N = b->nbf;
     p.boys = b->d_boys64;
     p.boys64_T = INFINITY;
+    p.prim_lt = kPrimKeepAll;
     e = launch_gen<double>(p, s);
   } else if (e == cudaSuccess) {
     CoopParams<double> p{};
@@ -188,6 +189,16 @@ static bool psplit_legal(const fsim_basis* b, int X, int Y, int ps) {
   return (ps == 1 || ps == 3 || ps == 9) && ps <= b->cls[X].ppmax;
 }
 
+int prim_threshold(double tau, bool fp32) {
+  if (!(tau > 0.0)) return kPrimKeepAll;
+  const double theta = fp32 ? std::min(std::ldexp(tau, -13), std::ldexp(1.0, -43))
+                            : std::min(std::ldexp(tau, -20), std::ldexp(1.0, -53));
+  if (!(theta > 0.0)) return kPrimKeepAll;  // underflow
+  int e = 0;
+  std::frexp(theta, &e);
+  return std::max(e - 1, kPrimKeepAll);  // 2^(e-1) <= theta
+}
+
 // Whether a build evaluates a class pair in FP64 with a CTA per quartet: the
 // heavy class pairs, and those with at most two waves of its CTAs, where the
 // unrolled kernel's threads, nine to a quartet, leave the FP64 pipes idle (six
@@ -246,6 +257,7 @@ int get_plan(fsim_basis* b, double tau, int shard, int nshards, int precision, F
       }
       FSIM_TRY(set_class_plan(b, X, Y, count, ps, coop, cp, cs, jk_flat_precision(precision)));
       cp.fp64 = precision == FSIM_DFLOAT && !dfloat_default(X, Y);
+      cp.prim_lt = prim_threshold(tau, precision == FSIM_MIXED);
       P->nquartets += cp.nquartets;
     }
   // class pairs with an f class: flattened screened (bra, ket) lists, one
@@ -259,6 +271,7 @@ int get_plan(fsim_basis* b, double tau, int shard, int nshards, int precision, F
       cp.nquartets = screened_counts(b, X, Y, tau, shard, nshards, count);
       FSIM_TRY(set_class_plan(b, X, Y, count, 1, 0, cp, 1, 1));
       cp.fp64 = precision == FSIM_DFLOAT;
+      cp.prim_lt = prim_threshold(tau, precision == FSIM_MIXED);
       P->nquartets += cp.nquartets;
     }
   *out = P;
@@ -289,6 +302,7 @@ static int launch_f_pair(fsim_basis* b, FockPlan* plan, int X, int Y, const Real
     p.K = Kacc;
     p.boys = std::is_same<Real, double>::value ? (const Real*)b->d_boys64 : (const Real*)b->d_boys32;
     p.boys64_T = boys64_T;
+    p.prim_lt = cp.prim_lt;
     const cudaError_t e = launch_gen<Real>(p, s);
     ++b->last_launches;
     if (e != cudaSuccess) {
@@ -361,6 +375,7 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
       p.K = Kacc;
       p.boys = b->d_boys64;
       p.boys64_T = boys64_T;
+      p.prim_lt = cp.prim_lt;
       return launch_gen<double>(p, s);
     }
   }
@@ -395,6 +410,7 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
   p.bra_ppmax = b->cls[X].ppmax;
   p.boys = quartet_boys<Real>(b);
   p.boys64_T = boys64_T;
+  p.prim_lt = cp.prim_lt;
   return dispatch_jk<Real>(X, Y, p, s);
 }
 
@@ -889,6 +905,7 @@ static int autotune_impl(fsim_basis* b, FockPlan* plan, const Real* Dr, float b6
       float best = 1e30f;
       Cand win = cands[0];
       ClassPairPlan tmp;
+      tmp.prim_lt = cp.prim_lt;
       for (const Cand& c : cands) {
         if ((rc = set_class_plan(b, X, Y, count, c.psplit, c.coop, tmp, c.csplit, jk_flat<Real>())) != FSIM_OK)
           break;

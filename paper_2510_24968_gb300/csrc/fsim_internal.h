@@ -67,6 +67,7 @@ struct DevClass {
   std::vector<int> h_npp;
   std::vector<double> h_Q;  // Schwarz bound of each pair, same order
   double* d_Q = nullptr;    // device copy of h_Q
+  uint4* ub = nullptr;      // bounds of the primitive pairs of each pair, same order (with h_Q; prim_mask)
   int nfield() const { return 4 + nnz; }
   template <typename Real>
   PairView<Real> view() const;
@@ -74,15 +75,15 @@ struct DevClass {
 
 template <>
 inline PairView<double> DevClass::view<double>() const {
-  return PairView<double>{n, ppmax, idx, npp, pd64, pq64};
+  return PairView<double>{n, ppmax, idx, npp, pd64, pq64, ub};
 }
 template <>
 inline PairView<float> DevClass::view<float>() const {
-  return PairView<float>{n, ppmax, idx, npp, pd32, pq32};
+  return PairView<float>{n, ppmax, idx, npp, pd32, pq32, ub};
 }
 template <>
 inline PairView<dfloat> DevClass::view<dfloat>() const {
-  return PairView<dfloat>{n, ppmax, idx, npp, pdx, pqx};
+  return PairView<dfloat>{n, ppmax, idx, npp, pdx, pqx, ub};
 }
 
 // Ket components per register chunk.  The per-thread registers of the unrolled
@@ -184,6 +185,7 @@ struct ClassPairPlan {
   int coop = 0;             // 1: table-driven kernel, a warp (FP32) or a CTA (FP64) per quartet
   int fp64 = 0;             // FSIM_DFLOAT plans: 1 = this class pair runs the FP64 kernel
   int tq = kJKThreads;      // kets per work item
+  int prim_lt = kPrimKeepAll;  // log2 of the primitive-quartet threshold
   int* d_prefix = nullptr;  // [nbra + 1]
   int* d_count = nullptr;   // [nbra]
 };
@@ -292,6 +294,8 @@ struct fsim_basis {
 };
 
 namespace fsim {
+// log2 of the primitive-quartet threshold of a build screened at tau (prim_mask)
+int prim_threshold(double tau, bool fp32);
 // the Boys table the quartet kernels of a precision stage (stage_boys)
 template <typename Real>
 inline const Real* quartet_boys(const fsim_basis* b) {

@@ -99,6 +99,9 @@ __global__ void __launch_bounds__(kGenThreads, 3) gen_kernel(GenParams<Real> P) 
   Real* sEk = reinterpret_cast<Real*>(gen_smem + Y.Ek);    // [nz][k], signed
   Real* sEb = reinterpret_cast<Real*>(gen_smem + Y.Eb);    // [nz][b]
   Real* sCoef = reinterpret_cast<Real*>(gen_smem + Y.coef);
+  int* sCol = reinterpret_cast<int*>(gen_smem + Y.col);    // [p]: bra << 8 | ket primitive pair
+  int* sBeg = sCol + Y.nbg * Y.nkg;                        // [b]: first p of bra primitive pair b of the group
+  int* sCnt = sBeg + 17;                                   // kept primitive quartets of each warp
   int* sPar = reinterpret_cast<int*>(gen_smem + Y.par);    // first parent | second << 10 | axis << 20 | coefficient << 22
   short* sSum = reinterpret_cast<short*>(gen_smem + Y.sum);  // [h'][h]: index of h + h'
   short* sNzc = reinterpret_cast<short*>(gen_smem + Y.nzc);  // h' | parity << 14
@@ -152,9 +155,32 @@ __global__ void __launch_bounds__(kGenThreads, 3) gen_kernel(GenParams<Real> P) 
       const int nb = min(Y.nbg, b_hi - b0);
       for (int k0 = 0; k0 < nppk; k0 += Y.nkg) {
         const int nk = min(Y.nkg, nppk - k0);
+        // the primitive quartets to evaluate, in order
+        int np;
+        {
+          const int b = tid / nk, k = k0 + tid % nk;
+          bool keep = false;
+          if (tid < nb * nk)
+            keep = P.prim_lt == kPrimKeepAll || prim_byte(P.ket.ub + j, k) >= prim_least(P.prim_lt, prim_byte(P.bra.ub + i, b0 + b));
+          const unsigned bal = __ballot_sync(0xffffffffu, keep);
+          if ((tid & 31) == 0) sCnt[tid >> 5] = __popc(bal);
+          __syncthreads();  // (also: the previous step's columns have been read)
+          int p = __popc(bal & ((1u << (tid & 31)) - 1u));
+          np = 0;
+          for (int w = 0; w < nth / 32; ++w) {
+            if (w < tid >> 5) p += sCnt[w];
+            np += sCnt[w];
+          }
+          if (tid < nb * nk) {
+            if (keep) sCol[p] = b << 8 | k;
+            if (tid % nk == 0) sBeg[b] = p;
+          }
+          if (tid == 0) sBeg[nb] = np;
+          __syncthreads();
+        }
         // 1. one primitive quartet per thread: sources and the in-place recursion
-        if (tid < nb * nk) {
-          const int b = b0 + tid / nk, k = k0 + tid % nk;
+        if (tid < np) {
+          const int b = b0 + (sCol[tid] >> 8), k = sCol[tid] & 255;
           const auto p4 = P.bra.pq[(size_t)b * P.bra.n + i];
           const Real p = p4.x, Px = p4.y, Py = p4.z, Pz = p4.w;
           const auto q4 = P.ket.pq[(size_t)k * P.ket.n + j];
@@ -197,7 +223,7 @@ __global__ void __launch_bounds__(kGenThreads, 3) gen_kernel(GenParams<Real> P) 
                   const Real a = ax == 0 ? X : (ax == 1 ? Yy : Z);
                   Real r;  // the branch is uniform: every thread is at the same h
                   if (h + x >= hi) break;
-                if (cf == 0) r = a * c1[x];
+                  if (cf == 0) r = a * c1[x];
                   else if (cf == 1) r = fma(a, c1[x], c2[x]);
                   else r = fma(a, c1[x], sCoef[cf] * c2[x]);
                   R[(h + x) * Y.npad] = r;
@@ -212,13 +238,14 @@ __global__ void __launch_bounds__(kGenThreads, 3) gen_kernel(GenParams<Real> P) 
         const int nW = C * nb * H1;
         for (int x = tid; x < nW; x += nth) {
           const int bh = x / H1, h = x - bh * H1, c = bh / nb, b = bh - c * nb;
-          const Real* Rp = sR + b * nk - k0;
+          const int p0 = sBeg[b], p1 = sBeg[b + 1];
           const short* sum = sSum + h;
           const int z0 = sOffc[c], z1 = sOffc[c + 1];
           Real& Wx = sW[(b * C + c) * H1 + h];
           Real acc = k0 == 0 ? Real(0) : Wx;
           if constexpr (std::is_same<Real, float>::value) {
-            for (int k = k0; k < k0 + nk; ++k) {
+            for (int p = p0; p < p1; ++p) {
+              const int k = sCol[p] & 255;
               Real part = Real(0);
               for (int z = z0; z < z1; ++z) {
                 const int w = sNzc[z], hz = w & 0x3fff;
@@ -229,24 +256,28 @@ __global__ void __launch_bounds__(kGenThreads, 3) gen_kernel(GenParams<Real> P) 
                   e = ldg_r(kp + (size_t)(4 + z) * kstride + (size_t)k * P.ket.n);
                   e = (w & 0x4000) ? -e : e;
                 }
-                part = fma(e, Rp[sum[hz * H1] * Y.npad + k], part);
+                part = fma(e, sR[sum[hz * H1] * Y.npad + p], part);
               }
               acc += part;
             }
           } else {
             for (int z = z0; z < z1; ++z) {
               const int w = sNzc[z], hz = w & 0x3fff;
-              const Real* Rz = Rp + sum[hz * H1] * Y.npad;
-              if (Y.stage_k) {
+              const Real* Rz = sR + sum[hz * H1] * Y.npad;
+              if (Y.stage_k && np == nb * nk) {  // nothing left out: no list to follow
+                const Real* E = sEk + z * nppk + k0 - p0;
+  #pragma unroll 3
+                for (int p = p0; p < p1; ++p) acc = fma(E[p], Rz[p], acc);
+              } else if (Y.stage_k) {
                 const Real* E = sEk + z * nppk;
   #pragma unroll 3
-                for (int k = k0; k < k0 + nk; ++k) acc = fma(E[k], Rz[k], acc);
+                for (int p = p0; p < p1; ++p) acc = fma(E[sCol[p] & 255], Rz[p], acc);
               } else {
                 const Real* E = kp + (size_t)(4 + z) * kstride;
                 const Real sg = (w & 0x4000) ? Real(-1) : Real(1);
                 Real part = Real(0);
   #pragma unroll 3
-                for (int k = k0; k < k0 + nk; ++k) part = fma(ldg_r(E + (size_t)k * P.ket.n), Rz[k], part);
+                for (int p = p0; p < p1; ++p) part = fma(ldg_r(E + (size_t)(sCol[p] & 255) * P.ket.n), Rz[p], part);
                 acc = fma(sg, part, acc);
               }
             }

@@ -7,16 +7,17 @@
 // weighted accumulators symmetrised by the caller).
 //
 // Layout of the work, for groups of nbg bra primitive pairs at a time:
-//   1. thread p < nbg * npp(ket) owns primitive quartet p: Boys function, sources,
-//      then the whole in-place R recursion in its own column of a shared-memory
-//      array R[h][p] (Eq. R-recursion from a table of parents; no barrier);
+//   1. thread p owns the p-th of the group's primitive quartets that can matter
+//      (prim_mask): Boys function, sources, then the whole in-place R recursion in
+//      its own column of a shared-memory array R[h][p] (Eq. R-recursion from a
+//      table of parents; no barrier);
 //   2. W[b][c][h] = sum_k sum_{h' in nz(c)} (-1)^{|h'|} E^{cd,k}_{c,h'} R[h + h'],
 //      elements over all threads with h fastest, so a warp shares c (and with
 //      it E, a broadcast) and the row of the sum table h + h';
 //   3. out[a][c] += sum_b sum_{h in nz(a)} E^{ab,b}_{a,h} W[b][c][h];
 // and per quartet the digestion: each thread sums one element of the J/K
 // blocks over the quartet block and adds it with one FP64 atomic.
-// Three barriers per group, none per primitive quartet or recursion level.  An
+// Five barriers per group, none per primitive quartet or recursion level.  An
 // FP64 launch with fewer quartets than resident CTAs shares each quartet's bra
 // primitive pairs out over several CTAs, which digest their partial blocks
 // (six (dd|dd) quartets: 0.77 ms with one CTA each).
@@ -43,7 +44,7 @@ struct GenLayout {
   int nbg, nkg;         // bra and ket primitive pairs per group (all of the ket's, but for the largest classes)
   int npad;             // row length of R: nbg * nkg, odd against bank conflicts
   int stage_k, stage_b; // E of the ket / bra pair staged in shared memory
-  unsigned R, W, out, Ek, Eb, coef, par, sum, nzc, nza, offc, offa, bytes;
+  unsigned R, W, out, Ek, Eb, coef, col, par, sum, nzc, nza, offc, offa, bytes;
 };
 
 template <typename Real>
@@ -63,6 +64,7 @@ struct GenParams {
   double* K;
   const Real* __restrict__ boys;     // full table, rows of kBoysCols
   float boys64_T;
+  int prim_lt;                       // log2 of the primitive-quartet threshold (prim_mask)
   GenLayout lay;                     // filled by launch_gen
 };
 
@@ -96,6 +98,7 @@ GenLayout gen_layout(int la, int lb, int lc, int ld, int ppb, int ppk) {
     y.Ek = take(y.stage_k ? (size_t)zc * ppk * sizeof(Real) : 0);
     y.Eb = take(y.stage_b ? (size_t)za * ppb * sizeof(Real) : 0);
     y.coef = take(16 * sizeof(Real));
+    y.col = take((size_t)(nbg * nkg + 16 + 8 + 1) * sizeof(int));
     y.par = take((size_t)NH * sizeof(int));
     y.sum = take((size_t)H1 * H2 * sizeof(short));
     y.nzc = take((size_t)zc * sizeof(short));

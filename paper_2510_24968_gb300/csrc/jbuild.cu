@@ -115,6 +115,7 @@ static int get_jplan(fsim_basis* b, double tau, int shard, int nshards, int prec
       for (int c : {3, 9})
         if (cp.nquartets * ps < target && c <= b->cls[X].ppmax) ps = c;
       FSIM_TRY(set_class_plan(b, X, Y, count, ps, 0, cp, 1, 0));
+      cp.prim_lt = prim_threshold(tau, precision == FSIM_MIXED);
       P->nquartets += cp.nquartets;
     }
   *out = P;
@@ -194,6 +195,7 @@ static int jeng_launch_all(fsim_basis* b, JPlan* plan, const Real* Dr, float b64
     p.bra_ppmax = b->cls[jb.X].ppmax;
     p.boys = boys;
     p.boys64_T = b64;
+    p.prim_lt = cp.prim_lt;
     ++b->last_launches;
     const cudaError_t e = dispatch_jeng<Real>(jb.X, jb.Y, p, st[k]);
     if (e != cudaSuccess) {

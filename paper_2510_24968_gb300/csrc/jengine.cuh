@@ -34,6 +34,7 @@ struct JEngParams {
   int bra_ppmax;
   const Real* __restrict__ boys;
   float boys64_T;
+  int prim_lt;                        // log2 of the primitive-quartet threshold (prim_mask)
 };
 
 // rho^{cd,k}[h'] for every pair j and primitive pair k of one class (one thread
@@ -118,12 +119,19 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
     if (q < tq && j < __ldg(P.ket_count + i)) {
       const int nppk = P.ket.npp[j];
       for (int b = bs; b < nppb; b += ps) {
+        unsigned todo = (1u << nppk) - 1u;
+        if constexpr (prim_skip<Real>(L)) {
+          todo = prim_mask(__ldg(P.ket.ub + j), prim_least(P.prim_lt, prim_byte(P.bra.ub + i, b)), nppk);
+          if (todo == 0) continue;
+        }
         const Real* sb = sbra + b * NFB;
         const Real p = sb[0], Px = sb[1], Py = sb[2], Pz = sb[3];
         Real jt[NH1];
 #pragma unroll
         for (int h = 0; h < NH1; ++h) jt[h] = Real(0);
-        for (int k = 0; k < nppk; ++k) {
+        while (todo != 0) {
+          const int k = __ffs(todo) - 1;
+          todo &= todo - 1;
           const auto q4 = P.ket.pq[(size_t)k * P.ket.n + j];
           const Real qq = q4.x;
           const Real X = Px - q4.y, Y = Py - q4.z, Z = Pz - q4.w;
