@@ -74,10 +74,21 @@ static cudaError_t launch_pair_data(int cls, int n, int ppmax, const int4* idx, 
 }
 
 // (Re)build the device data of pair class `cls` in the given pair order.
+// E non-zeros of the FP32 pair data by fours: the quartet kernels load a ket's in
+// 16-byte words.  One thread per (group of four, primitive pair, pair).
+__global__ void pair_quads_kernel(int nnz, size_t fs, const float* __restrict__ pd, float4* __restrict__ pe) {
+  const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int g = (int)(x / fs);
+  if (4 * g >= nnz) return;
+  float e[4];
+  for (int i = 0; i < 4; ++i) e[i] = 4 * g + i < nnz ? pd[(size_t)(4 + 4 * g + i) * fs + x % fs] : 0.0f;
+  pe[x] = make_float4(e[0], e[1], e[2], e[3]);
+}
+
 int build_pair_data(fsim_basis* b, int cls, const std::vector<int4>& order) {
   DevClass& C = b->cls[cls];
   dev_free(C.idx); dev_free(C.npp); dev_free(C.pd64); dev_free(C.pd32); dev_free(C.pq64); dev_free(C.pq32);
-  dev_free(C.pdx); dev_free(C.pqx);
+  dev_free(C.pe32); dev_free(C.pdx); dev_free(C.pqx);
   b->dfloat_ready = false;  // the double-float copies follow the pair order; remade on next use
   C.n = (int)order.size();
   C.nnz = pair_cls_nnz(cls);
@@ -95,9 +106,14 @@ int build_pair_data(fsim_basis* b, int cls, const std::vector<int4>& order) {
   FSIM_TRY(dev_alloc(&C.pd32, (size_t)C.nfield() * C.ppmax * C.n));
   FSIM_TRY(dev_alloc(&C.pq64, (size_t)C.ppmax * C.n));
   FSIM_TRY(dev_alloc(&C.pq32, (size_t)C.ppmax * C.n));
+  const size_t fs = (size_t)C.ppmax * C.n;
+  const size_t quads = cls < kNumPairCls ? (size_t)((C.nnz + 3) / 4) * fs : 0;  // (the kernel of f shells does not read them)
+  if (quads) FSIM_TRY(dev_alloc(&C.pe32, quads));
   FSIM_CK(cudaMemcpy(C.idx, order.data(), sizeof(int4) * C.n, cudaMemcpyHostToDevice));
   FSIM_CK(cudaMemcpy(C.npp, C.h_npp.data(), sizeof(int) * C.n, cudaMemcpyHostToDevice));
   FSIM_CK(launch_pair_data(cls, C.n, C.ppmax, C.idx, b, C.pd64, C.pd32, C.pq64, C.pq32));
+  if (quads) pair_quads_kernel<<<(unsigned)((quads + 255) / 256), 256>>>(C.nnz, fs, C.pd32, C.pe32);
+  FSIM_CK(cudaGetLastError());
   return FSIM_OK;
 }
 
@@ -507,7 +523,7 @@ void fsim_basis_destroy(fsim_basis* b) {
   if (!b) return;
   for (auto& C : b->cls) {
     dev_free(C.idx); dev_free(C.npp); dev_free(C.pd64); dev_free(C.pd32); dev_free(C.pq64); dev_free(C.pq32);
-    dev_free(C.pdx); dev_free(C.pqx); dev_free(C.d_Q); dev_free(C.ub);
+    dev_free(C.pe32); dev_free(C.pdx); dev_free(C.pqx); dev_free(C.d_Q); dev_free(C.ub);
   }
   for (auto* p : b->plans) {
     for (auto& row : p->cp)

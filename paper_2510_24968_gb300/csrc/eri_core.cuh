@@ -54,6 +54,7 @@ struct PairView {
   const int* __restrict__ npp;                      // primitive pairs of each pair
   const Real* __restrict__ pd;                      // [field][pp][pair]
   const typename Vec4<Real>::type* __restrict__ pq;  // (p, Px, Py, Pz) at [pp][pair]
+  const float4* __restrict__ pe4;                    // FP32: E non-zeros by fours, [z / 4][pp][pair]
   const uint4* __restrict__ ub;                      // Schwarz bounds of the pair's primitive pairs (prim_mask)
 };
 
@@ -238,6 +239,30 @@ struct KetChunks {
   }
 };
 
+// How the FP32 kernel of a class pair loads its kets' data.  Two warps a scheduler
+// do not hide a load's latency (a quarter of the stalls of the middle orders), and
+// a chunk's E non-zeros were loads of 4 bytes with an address each.
+//   kNext: (q, Q) of the next primitive quartet is loaded while this one is evaluated;
+//   kEarly: so is this one's single E, before the Boys function;
+//   kQuads: the E non-zeros come in 16-byte loads;
+//   kTouch: these are prefetched into L1 before the Boys function.
+// By class pair, from timing each form of all 21 on clouds of 12 and 20 atoms
+// (change of the kernel's time, 20 atoms): ket ss with kEarly -24 % (pp bra) to -10
+// % (dd), but +5 % (ss); quads with kTouch (pp|ps) -4, (pp|pp) -11, (ds|pp) -12 %;
+// without it (dp|ps) -13, (dp|pp) -9, (dp|dp) -5 %, where the prefetches'
+// addresses cost registers.  The small kernels, whose other warps hide the loads,
+// and bra dd, whose 16-byte loads spill ((dd|dd) +17 %), keep the plain loads.
+// 20-atom cloud, whole build: 134.5 -> 125.1 ms.
+template <typename Real, int LA, int LB, int LC, int LD>
+struct KetLoads {
+  static constexpr bool dd = LA == 2 && LB == 2, dp = LA == 2 && LB == 1;
+  static constexpr bool kEarly = std::is_same<Real, float>::value && LC == 0 && LA + LB >= 2;
+  static constexpr bool kQuads = std::is_same<Real, float>::value && LC > 0 && LA + LB + LC + LD >= 3 &&
+                                 (!dd || LD == 0);
+  static constexpr bool kTouch = kQuads && !dp && !(dd && LC == 2);
+  static constexpr bool kNext = kEarly || kQuads;
+};
+
 // Contracted quartet block for one ket chunk: out(a, cs) for all bra components
 // a and ket components c = ch*CS + cs < NC, accumulated in this thread's
 // shared-memory slots so[(a * CS + cs) * kJKThreads] (so the registers hold
@@ -269,10 +294,20 @@ __device__ __forceinline__ void quartet_chunk(Real* __restrict__ so, const BraAt
   constexpr int NH1 = BC::NH;
   constexpr int NZM = KCh::max_nnz();
   constexpr bool kSkip = prim_skip<Real>(L);
+  using KL = KetLoads<Real, LA, LB, LC, LD>;
 #pragma unroll
   for (int x = 0; x < BC::NC * CS; ++x) so[x * kJKThreads] = Real(0);
   const size_t kstride = (size_t)ket.ppmax * ket.n;
   const int ks = (bstep + nppb - 1) / nppb;
+  int touch0 = 0, ntouch = 0;  // the chunk's groups of four E non-zeros
+  if constexpr (KL::kTouch)
+    static_for<KCh::NCH>([&](auto Ch) {
+      constexpr int CH = decltype(Ch)::value;
+      if (ch == CH) {
+        touch0 = KC::off(CH * CS) / 4;
+        ntouch = (KC::off(CH * CS) + KCh::nnz_of(CH) + 3) / 4 - touch0;
+      }
+    });
   for (int u = b0; u < nppb * ks; u += bstep) {
     const int b = u % nppb;
     // the ket primitive pairs to take with this bra primitive pair: every ks-th from u / nppb
@@ -290,11 +325,25 @@ __device__ __forceinline__ void quartet_chunk(Real* __restrict__ so, const BraAt
     for (int h = 0; h < NH1; ++h)
 #pragma unroll
       for (int cs = 0; cs < CS; ++cs) W[h][cs] = Real(0);
-    for (int k = kSkip ? __ffs(todo) - 1 : u / nppb; kSkip ? todo != 0 : k < nppk;
-         k = kSkip ? __ffs(todo) - 1 : k + ks) {
+    int k = kSkip ? __ffs(todo) - 1 : u / nppb;
+    typename Vec4<Real>::type qn;
+    if constexpr (KL::kNext) qn = ket.pq[(size_t)min(k, nppk - 1) * ket.n + j];
+    while (kSkip ? todo != 0 : k < nppk) {
       todo &= todo - 1;
       const Real* kp = ket.pd + (size_t)k * ket.n + j;
-      const auto q4 = ket.pq[(size_t)k * ket.n + j];
+      const float4* ke = ket.pe4 + (size_t)k * ket.n + j;
+      typename Vec4<Real>::type q4;
+      if constexpr (KL::kNext) q4 = qn; else q4 = ket.pq[(size_t)k * ket.n + j];
+      k = kSkip ? __ffs(todo) - 1 : k + ks;
+      if constexpr (KL::kNext)
+        if (kSkip ? todo != 0 : k < nppk) qn = ket.pq[(size_t)k * ket.n + j];
+      if constexpr (KL::kTouch) {
+#pragma unroll
+        for (int g = 0; g < NZM / 4 + 2; ++g)
+          if (g < ntouch) asm volatile("prefetch.global.L1 [%0];" ::"l"(ke + (size_t)(touch0 + g) * kstride));
+      }
+      Real E0;
+      if constexpr (KL::kEarly) E0 = ldg_r(kp + 4 * kstride);
       const Real q = q4.x, Qx = q4.y, Qy = q4.z, Qz = q4.w;
       const Real X = Px - Qx, Y = Py - Qy, Z = Pz - Qz;
       Real src[L + 1];
@@ -308,8 +357,22 @@ __device__ __forceinline__ void quartet_chunk(Real* __restrict__ so, const BraAt
         constexpr int c0 = CH * CS;
         constexpr int nzoff = KC::off(c0);
         constexpr int NZ = KCh::nnz_of(CH);
+        if constexpr (KL::kQuads) {
 #pragma unroll
-        for (int z = 0; z < NZ; ++z) Ek[z] = ldg_r(kp + (size_t)(4 + nzoff + z) * kstride);
+          for (int g = nzoff / 4; g < (nzoff + NZ + 3) / 4; ++g) {
+            const float4 e4 = __ldg(ke + (size_t)g * kstride);
+            const float e[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+              if (4 * g + x >= nzoff && 4 * g + x < nzoff + NZ) Ek[4 * g + x - nzoff] = e[x];
+          }
+        } else if constexpr (KL::kEarly) {
+          static_assert(KC::NNZ == 1, "one E non-zero");
+          Ek[0] = E0;
+        } else {
+#pragma unroll
+          for (int z = 0; z < NZ; ++z) Ek[z] = ldg_r(kp + (size_t)(4 + nzoff + z) * kstride);
+        }
         static_for<CS>([&](auto Cs) {
           constexpr int cs = decltype(Cs)::value;
           constexpr int c = c0 + cs;

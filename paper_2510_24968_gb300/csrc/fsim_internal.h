@@ -61,6 +61,7 @@ struct DevClass {
   float* pd32 = nullptr;
   double4_32a* pq64 = nullptr;  // (p, P) at [ppmax][n]
   float4* pq32 = nullptr;
+  float4* pe32 = nullptr;   // E non-zeros of pd32 by fours, [ceil(nnz / 4)][ppmax][n]
   dfloat* pdx = nullptr;    // double-float copies of pd64 / pq64 (made on first FSIM_DFLOAT use)
   dfloat4* pqx = nullptr;
   std::vector<int4> h_idx;  // host copy, same order
@@ -75,15 +76,15 @@ struct DevClass {
 
 template <>
 inline PairView<double> DevClass::view<double>() const {
-  return PairView<double>{n, ppmax, idx, npp, pd64, pq64, ub};
+  return PairView<double>{n, ppmax, idx, npp, pd64, pq64, nullptr, ub};
 }
 template <>
 inline PairView<float> DevClass::view<float>() const {
-  return PairView<float>{n, ppmax, idx, npp, pd32, pq32, ub};
+  return PairView<float>{n, ppmax, idx, npp, pd32, pq32, pe32, ub};
 }
 template <>
 inline PairView<dfloat> DevClass::view<dfloat>() const {
-  return PairView<dfloat>{n, ppmax, idx, npp, pdx, pqx, ub};
+  return PairView<dfloat>{n, ppmax, idx, npp, pdx, pqx, nullptr, ub};
 }
 
 // Ket components per register chunk.  The per-thread registers of the unrolled
