@@ -143,7 +143,8 @@ static int jeng_launch_all(fsim_basis* b, JPlan* plan, const Real* Dr, float b64
     const DevClass& C = b->cls[Y];
     if (C.n == 0) continue;
     Real*& rho = rho_buf<Real>(b, Y);
-    if (!rho) FSIM_TRY(dev_alloc(&rho, (size_t)nherm(pair_cls_la(Y) + pair_cls_lb(Y)) * C.ppmax * C.n));
+    const int nh = nherm(pair_cls_la(Y) + pair_cls_lb(Y));  // (a multiple of four for the 16-byte loads)
+    if (!rho) FSIM_TRY(dev_alloc(&rho, (size_t)((nh + 3) / 4 * 4) * C.ppmax * C.n));
     const cudaError_t e = dispatch_rho<Real>(Y, C.view<Real>(), Dr, b->nbf, rho, s);
     if (e != cudaSuccess) {
       set_error("J-engine density vectors (%d): %s", Y, cudaGetErrorString(e));

@@ -37,8 +37,19 @@ struct JEngParams {
   int prim_lt;                        // log2 of the primitive-quartet threshold (prim_mask)
 };
 
+// How the FP32 kernels load a ket's data (as KetLoads of eri_core.cuh, for the same
+// reason): rho by fours in 16-byte loads and (q, Q) of the next primitive pair a step
+// ahead, but for kets of two s shells, whose one rho gains nothing ((ss|ss) +6 %);
+// prefetches into L1 where the bra has pp or more ((pp|pp) 69.4 -> 54.2 us of
+// (H2O)_8 with, 59.0 without; (ss|pp) 72.1 -> 64.8 without, 72.1 with).  12-atom
+// cloud, J alone: 11.48 -> 10.65 ms.
+template <typename Real, int LC>
+constexpr bool jeng_quads() { return std::is_same<Real, float>::value && LC > 0; }
+template <typename Real, int LA, int LB, int LC>
+constexpr bool jeng_touch() { return jeng_quads<Real, LC>() && LA + LB >= 2; }
+
 // rho^{cd,k}[h'] for every pair j and primitive pair k of one class (one thread
-// each): rho[(h' * ppmax + k) * n + j].
+// each): rho[(h' * ppmax + k) * n + j], or by fours [h' / 4][k][j][h' % 4] (jeng_quads).
 template <typename Real, int LC, int LD>
 __global__ void jeng_rho_kernel(PairView<Real> ket, const Real* __restrict__ D, int N, Real* __restrict__ rho) {
   using KC = PairCls<LC, LD>;
@@ -67,7 +78,10 @@ __global__ void jeng_rho_kernel(PairView<Real> ket, const Real* __restrict__ D, 
     for (int h = 0; h < KC::NH; ++h) acc[h] = deg * acc[h];
   }
 #pragma unroll
-  for (int h = 0; h < KC::NH; ++h) rho[((size_t)h * ket.ppmax + k) * ket.n + j] = acc[h];
+  for (int h = 0; h < KC::NH; ++h) {
+    if constexpr (jeng_quads<Real, LC>()) rho[((((size_t)(h / 4) * ket.ppmax + k) * ket.n + j) << 2) + (h & 3)] = acc[h];
+    else rho[((size_t)h * ket.ppmax + k) * ket.n + j] = acc[h];
+  }
 }
 
 template <typename Real, int LA, int LB>
@@ -92,6 +106,7 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
   constexpr int NFB = 4 + BC::NNZ;
   constexpr int BK = Boys<Real>::NCOL;
   constexpr int NWARP = kJKThreads / 32;
+  constexpr bool kQuads = jeng_quads<Real, LC>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* sBoys = reinterpret_cast<Real*>(smem_raw);
   Real* sJ = reinterpret_cast<Real*>(smem_raw + (jk_boys_smem<Real>() + 15) / 16 * 16);  // [a][thread]
@@ -129,20 +144,39 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
         Real jt[NH1];
 #pragma unroll
         for (int h = 0; h < NH1; ++h) jt[h] = Real(0);
+        int k = __ffs(todo) - 1;
+        typename Vec4<Real>::type qn;
+        if constexpr (kQuads) qn = P.ket.pq[(size_t)k * P.ket.n + j];
         while (todo != 0) {
-          const int k = __ffs(todo) - 1;
           todo &= todo - 1;
-          const auto q4 = P.ket.pq[(size_t)k * P.ket.n + j];
+          const Real* rk = P.rho + (size_t)k * P.ket.n + j;
+          const float4* rk4 = reinterpret_cast<const float4*>(P.rho) + (size_t)k * P.ket.n + j;
+          typename Vec4<Real>::type q4;
+          if constexpr (kQuads) q4 = qn; else q4 = P.ket.pq[(size_t)k * P.ket.n + j];
+          k = __ffs(todo) - 1;
+          if constexpr (kQuads)
+            if (todo != 0) qn = P.ket.pq[(size_t)k * P.ket.n + j];
+          if constexpr (jeng_touch<Real, LA, LB, LC>()) {
+#pragma unroll
+            for (int g = 0; g < (NH2 + 3) / 4; ++g)
+              asm volatile("prefetch.global.L1 [%0];" ::"l"(rk4 + (size_t)g * kstride));
+          }
           const Real qq = q4.x;
           const Real X = Px - q4.y, Y = Py - q4.z, Z = Pz - q4.w;
           Real src[L + 1];
           prim_sources<Real, L>(p, qq, X, Y, Z, src, sBoys, BK, P.boys64_T);
           Real R[NH];
           hermite_R<Real, L>(R, src, X, Y, Z);
-          const Real* rk = P.rho + (size_t)k * P.ket.n + j;
+          float4 r4;
           static_for<NH2>([&](auto Hk) {
             constexpr int hk = decltype(Hk)::value;
-            const Real r = ldg_r(rk + (size_t)hk * kstride);
+            Real r;
+            if constexpr (kQuads) {
+              if constexpr (hk % 4 == 0) r4 = __ldg(rk4 + (size_t)(hk / 4) * kstride);
+              r = hk % 4 == 0 ? r4.x : (hk % 4 == 1 ? r4.y : (hk % 4 == 2 ? r4.z : r4.w));
+            } else {
+              r = ldg_r(rk + (size_t)hk * kstride);
+            }
             static_for<NH1>([&](auto Hb) {
               constexpr int hb = decltype(Hb)::value;
               constexpr int hr = hidx(herm_t(hb) + herm_t(hk), herm_u(hb) + herm_u(hk), herm_v(hb) + herm_v(hk));
