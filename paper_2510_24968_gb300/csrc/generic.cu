@@ -85,7 +85,7 @@ constexpr GenTables make_gen_tables() {
 __device__ const GenTables kGenTables = make_gen_tables();
 
 template <typename Real>
-__global__ void __launch_bounds__(kGenThreads, 3) gen_kernel(GenParams<Real> P) {
+__global__ void __launch_bounds__(kGenThreads, 4) gen_kernel(GenParams<Real> P) {
   extern __shared__ __align__(16) unsigned char gen_smem[];
   const GenLayout& Y = P.lay;
   const int la = P.la, lb = P.lb, lc = P.lc, ld = P.ld;

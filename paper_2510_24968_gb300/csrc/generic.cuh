@@ -29,6 +29,9 @@
 // evaluated once, and no thread holds a quartet-sized array.  The unrolled
 // kernel of eri_core.cuh repeats R for every ket chunk and, at one warp per
 // scheduler, waits on its local-memory arrays: it used 50-65 % of the FP64 pipe.
+// 64 registers a thread let a fourth CTA onto the SM where its shared memory fits,
+// to fill the others' barriers ((H2O)_8 FP64 48.1 -> 47.3 ms, f shells 18.0 -> 16.8);
+// groups cut down so that four always fit gain nothing more (47.7, 17.0).
 #pragma once
 #include "eri_core.cuh"
 
