@@ -22,6 +22,7 @@
 #include <cstring>
 #include <vector>
 
+#include "fork_join.h"
 #include "fsim_internal.h"
 
 namespace fsim {
@@ -230,23 +231,16 @@ int launch_batch(fsim_batch* bt, int prec, cudaStream_t s, bool dry) {
   std::stable_sort(order.begin(), order.end(), [&](const std::pair<int, int>& a, const std::pair<int, int>& c) {
     return bt->cp[prec][a.first][a.second].cost > bt->cp[prec][c.first][c.second].cost;
   });
-  constexpr int NS = fsim_batch::kAux + 1;
-  cudaStream_t st[NS] = {s};
-  for (int k = 0; k < fsim_batch::kAux; ++k) st[k + 1] = bt->aux[k];
-  double load[NS] = {};
-  if (!dry) {
-    FSIM_CK(cudaEventRecord(bt->fork_ev, s));
-    for (int k = 1; k < NS; ++k) FSIM_CK(cudaStreamWaitEvent(st[k], bt->fork_ev, 0));
-  }
   int rc = FSIM_OK;
-  for (const auto& [X, Y] : order) {
-    const fsim_batch::CPB& C = bt->cp[prec][X][Y];
-    int k = 0;
-    for (int t = 1; t < NS; ++t)
-      if (load[t] < load[k]) k = t;
-    load[k] += C.cost;
-    cudaError_t e = cudaSuccess;
-    {
+  auto launches = [&](const cudaStream_t* st) {
+    constexpr int NS = fsim_batch::kAux + 1;
+    double load[NS] = {};
+    for (const auto& [X, Y] : order) {
+      const fsim_batch::CPB& C = bt->cp[prec][X][Y];
+      int k = 0;
+      for (int t = 1; t < NS; ++t)
+        if (load[t] < load[k]) k = t;
+      load[k] += C.cost;
       JKParams<Real> p{};
       p.mols = (const JKMol<Real>*)C.d_mols;
       p.mol_prefix = C.d_prefix;
@@ -262,20 +256,22 @@ int launch_batch(fsim_batch* bt, int prec, cudaStream_t s, bool dry) {
       p.bra_ppmax = C.bra_ppmax;
       p.boys = quartet_boys<Real>(bt->b[0]);
       p.boys64_T = INFINITY;
-      e = dispatch<Real>(X, Y, p, st[k]);
+      const cudaError_t e = dispatch<Real>(X, Y, p, st[k]);
+      if (e != cudaSuccess) {
+        set_error("batched J/K (%d|%d): %s", X, Y, cudaGetErrorString(e));
+        rc = FSIM_ECUDA;
+        return;
+      }
     }
-    if (e != cudaSuccess) {
-      set_error("batched J/K (%d|%d): %s", X, Y, cudaGetErrorString(e));
-      rc = FSIM_ECUDA;
-      break;
-    }
+  };
+  if (dry) {
+    const cudaStream_t st[fsim_batch::kAux + 1] = {s, bt->aux[0], bt->aux[1], bt->aux[2]};
+    launches(st);
+    return rc;
   }
-  if (dry) return rc;
-  for (int k = 1; k < NS; ++k) {  // after an error too: no stream is left unjoined
-    FSIM_CK(cudaEventRecord(bt->join_ev[k - 1], st[k]));
-    FSIM_CK(cudaStreamWaitEvent(s, bt->join_ev[k - 1], 0));
-  }
-  if (rc != FSIM_OK) return rc;
+  const cudaError_t fe = fork_join(s, fsim_batch::kAux, bt->aux, bt->fork_ev, bt->join_ev, launches);
+  FSIM_TRY(rc);
+  FSIM_CK(fe);
   dim3 g2(std::max(1, std::min(64, (bt->maxN * bt->maxN + 255) / 256)), bt->nmol);
   batch_symmetrize_kernel<<<g2, 256, 0, s>>>(bt->d_ptrs, bt->d_active);
   FSIM_CK(cudaGetLastError());

@@ -12,6 +12,7 @@
 #include <cstring>
 
 #include "coop.cuh"
+#include "fork_join.h"
 #include "fsim_internal.h"
 #include "generic.cuh"
 
@@ -464,34 +465,32 @@ static int launch_all(fsim_basis* b, FockPlan* plan, const Real* Dr, float boys6
         if (plan->cp[X][Y].nquartets > 0)
           jobs.push_back(Job{X, Y, (double)plan->cp[X][Y].nquartets * class_cost(X, Y)});
     std::stable_sort(jobs.begin(), jobs.end(), [](const Job& a, const Job& c) { return a.cost > c.cost; });
-    constexpr int NS = fsim_basis::kAuxStreams + 1;
-    cudaStream_t st[NS] = {s};
-    for (int k = 0; k < fsim_basis::kAuxStreams; ++k) st[k + 1] = b->aux[k];
-    const int nuse = std::min<int>(NS, (int)jobs.size());
-    FSIM_CK(cudaEventRecord(b->fork_ev, s));
-    for (int k = 1; k < nuse; ++k) FSIM_CK(cudaStreamWaitEvent(st[k], b->fork_ev, 0));
-    double load[NS] = {};
-    for (const Job& j : jobs) {
-      int k = 0;
-      for (int t = 1; t < nuse; ++t)
-        if (load[t] < load[k]) k = t;
-      load[k] += j.cost;
-      if (j.X >= kNumPairCls) {
-        FSIM_TRY(launch_f_pair<Real>(b, plan, j.X, j.Y, Dr, boys64_T, b->d_Jacc, b->d_Kacc, st[k], D64));
-        continue;
+    const int nuse = std::min<int>(fsim_basis::kAuxStreams + 1, (int)jobs.size());
+    double load[fsim_basis::kAuxStreams + 1] = {};
+    int rc = FSIM_OK;
+    const cudaError_t fe = fork_join(s, std::max(nuse - 1, 0), b->aux, b->fork_ev, b->join_ev, [&](const cudaStream_t* st) {
+      for (const Job& j : jobs) {
+        int k = 0;
+        for (int t = 1; t < nuse; ++t)
+          if (load[t] < load[k]) k = t;
+        load[k] += j.cost;
+        if (j.X >= kNumPairCls) {
+          rc = launch_f_pair<Real>(b, plan, j.X, j.Y, Dr, boys64_T, b->d_Jacc, b->d_Kacc, st[k], D64);
+          if (rc != FSIM_OK) return;
+          continue;
+        }
+        ++b->last_launches;
+        const cudaError_t e = launch_cp<Real>(b, j.X, j.Y, plan->cp[j.X][j.Y], Dr, b->d_Jacc, b->d_Kacc, boys64_T,
+                                              st[k], D64);
+        if (e != cudaSuccess) {
+          set_error("J/K kernel (%d|%d): %s", j.X, j.Y, cudaGetErrorString(e));
+          rc = FSIM_ECUDA;
+          return;
+        }
       }
-      ++b->last_launches;
-      const cudaError_t e = launch_cp<Real>(b, j.X, j.Y, plan->cp[j.X][j.Y], Dr, b->d_Jacc, b->d_Kacc, boys64_T,
-                                            st[k], D64);
-      if (e != cudaSuccess) {
-        set_error("J/K kernel (%d|%d): %s", j.X, j.Y, cudaGetErrorString(e));
-        return FSIM_ECUDA;
-      }
-    }
-    for (int k = 1; k < nuse; ++k) {
-      FSIM_CK(cudaEventRecord(b->join_ev[k - 1], st[k]));
-      FSIM_CK(cudaStreamWaitEvent(s, b->join_ev[k - 1], 0));
-    }
+    });
+    FSIM_TRY(rc);
+    FSIM_CK(fe);
     return FSIM_OK;
   }
   FSIM_TRY(launch_f_pairs<Real>(b, plan, Dr, boys64_T, b->d_Jacc, b->d_Kacc, s, D64));

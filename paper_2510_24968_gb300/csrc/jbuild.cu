@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "fork_join.h"
 #include "fsim_internal.h"
 #include "jengine.cuh"
 
@@ -169,45 +170,42 @@ static int jeng_launch_all(fsim_basis* b, JPlan* plan, const Real* Dr, float b64
       jobs.push_back(Job{X, Y, (double)cp.nquartets * per});
     }
   std::stable_sort(jobs.begin(), jobs.end(), [](const Job& a, const Job& c) { return a.cost > c.cost; });
-  constexpr int NS = fsim_basis::kAuxStreams + 1;
-  cudaStream_t st[NS] = {s};
-  for (int k = 0; k < fsim_basis::kAuxStreams; ++k) st[k + 1] = b->aux[k];
-  const int nuse = std::min<int>(NS, (int)jobs.size());
-  FSIM_CK(cudaEventRecord(b->fork_ev, s));
-  for (int k = 1; k < nuse; ++k) FSIM_CK(cudaStreamWaitEvent(st[k], b->fork_ev, 0));
-  double load[NS] = {};
+  const int nuse = std::min<int>(fsim_basis::kAuxStreams + 1, (int)jobs.size());
+  double load[fsim_basis::kAuxStreams + 1] = {};
   const Real* boys = quartet_boys<Real>(b);
-  for (const Job& jb : jobs) {
-    int k = 0;
-    for (int t = 1; t < nuse; ++t)
-      if (load[t] < load[k]) k = t;
-    load[k] += jb.cost;
-    const ClassPairPlan& cp = plan->cp[jb.X][jb.Y];
-    JEngParams<Real> p{};
-    p.bra = b->cls[jb.X].view<Real>();
-    p.ket = b->cls[jb.Y].view<Real>();
-    p.rho = rho_buf<Real>(b, jb.Y);
-    p.prefix = cp.d_prefix;
-    p.ket_count = cp.d_count;
-    p.N = b->nbf;
-    p.J = b->d_Jacc;
-    p.nitems = cp.nitems;
-    p.psplit = cp.psplit;
-    p.bra_ppmax = b->cls[jb.X].ppmax;
-    p.boys = boys;
-    p.boys64_T = b64;
-    p.prim_lt = cp.prim_lt;
-    ++b->last_launches;
-    const cudaError_t e = dispatch_jeng<Real>(jb.X, jb.Y, p, st[k]);
-    if (e != cudaSuccess) {
-      set_error("J-engine kernel (%d|%d): %s", jb.X, jb.Y, cudaGetErrorString(e));
-      return FSIM_ECUDA;
+  int rc = FSIM_OK;
+  const cudaError_t fe = fork_join(s, std::max(nuse - 1, 0), b->aux, b->fork_ev, b->join_ev, [&](const cudaStream_t* st) {
+    for (const Job& jb : jobs) {
+      int k = 0;
+      for (int t = 1; t < nuse; ++t)
+        if (load[t] < load[k]) k = t;
+      load[k] += jb.cost;
+      const ClassPairPlan& cp = plan->cp[jb.X][jb.Y];
+      JEngParams<Real> p{};
+      p.bra = b->cls[jb.X].view<Real>();
+      p.ket = b->cls[jb.Y].view<Real>();
+      p.rho = rho_buf<Real>(b, jb.Y);
+      p.prefix = cp.d_prefix;
+      p.ket_count = cp.d_count;
+      p.N = b->nbf;
+      p.J = b->d_Jacc;
+      p.nitems = cp.nitems;
+      p.psplit = cp.psplit;
+      p.bra_ppmax = b->cls[jb.X].ppmax;
+      p.boys = boys;
+      p.boys64_T = b64;
+      p.prim_lt = cp.prim_lt;
+      ++b->last_launches;
+      const cudaError_t e = dispatch_jeng<Real>(jb.X, jb.Y, p, st[k]);
+      if (e != cudaSuccess) {
+        set_error("J-engine kernel (%d|%d): %s", jb.X, jb.Y, cudaGetErrorString(e));
+        rc = FSIM_ECUDA;
+        return;
+      }
     }
-  }
-  for (int k = 1; k < nuse; ++k) {
-    FSIM_CK(cudaEventRecord(b->join_ev[k - 1], st[k]));
-    FSIM_CK(cudaStreamWaitEvent(s, b->join_ev[k - 1], 0));
-  }
+  });
+  FSIM_TRY(rc);
+  FSIM_CK(fe);
   return FSIM_OK;
 }
 
