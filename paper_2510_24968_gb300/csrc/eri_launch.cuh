@@ -20,7 +20,10 @@ cudaError_t launch_jk(const JKParams<Real>& p, cudaStream_t s) {
                 "per-thread quartet blocks exceed the shared-memory budget");
   auto k = jk_kernel<Real, LA, LB, LC, LD, CS>;
   const size_t smem = jk_smem_bytes<Real, LA, LB, CS>(p.bra_ppmax);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the kernel's limit belongs to the process: always the largest any handle needs,
+  // so that another thread's launch with fewer primitives cannot lower it in between
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)jk_smem_bytes<Real, LA, LB, CS>(kMaxPrim * kMaxPrim));
   if (e != cudaSuccess) return e;
   if (p.nitems == 0) return cudaSuccess;
   int occ = 0;

@@ -367,7 +367,9 @@ cudaError_t launch_gen(const GenParams<Real>& in, cudaStream_t s) {
   GenParams<Real> p = in;
   p.lay = gen_layout<Real>(p.la, p.lb, p.lc, p.ld, p.bra.ppmax, p.ket.ppmax);
   const size_t smem = p.lay.bytes;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // one kernel for every class pair and the limit is the process's: always the
+  // largest layout, so that no other thread's launch can lower it in between
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGenMaxSmem);
   if (e != cudaSuccess || p.nitems == 0) return e;
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kGenThreads, smem);

@@ -41,6 +41,7 @@ constexpr int kGenThreads = 256;
 constexpr int kGenMaxL = 12;     // (ff|ff)
 constexpr int kGenMaxH1 = nherm(6);  // Hermite terms of an (f f) pair
 constexpr int kGenMaxNC = 100;       // components of an (f f) pair
+constexpr unsigned kGenMaxSmem = 226 * 1024;  // no layout is larger
 
 // Shared-memory layout of a class pair (byte offsets).
 struct GenLayout {
@@ -80,7 +81,7 @@ GenLayout gen_layout(int la, int lb, int lc, int ld, int ppb, int ppk) {
   const int L = la + lb + lc + ld, H1 = nherm(la + lb), H2 = nherm(lc + ld), NH = nherm(L);
   const int A = ncart(la) * ncart(lb), C = ncart(lc) * ncart(ld);
   const int za = gen_pair_nnz(la, lb), zc = gen_pair_nnz(lc, ld);
-  constexpr unsigned kThree = 74 * 1024, kMax = 226 * 1024, kStage = 16 * 1024;
+  constexpr unsigned kThree = 74 * 1024, kStage = 16 * 1024;
   int nkg = ppk;
   auto make = [&](int nbg) {
     GenLayout y{};
@@ -112,7 +113,7 @@ GenLayout gen_layout(int la, int lb, int lc, int ld, int ppb, int ppk) {
     return y;
   };
   GenLayout best = make(1);
-  while (best.bytes > kMax && nkg > 1) {
+  while (best.bytes > kGenMaxSmem && nkg > 1) {
     nkg = (nkg + 1) / 2;
     best = make(1);
   }

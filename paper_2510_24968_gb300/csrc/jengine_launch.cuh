@@ -14,7 +14,9 @@ cudaError_t launch_jeng(const JEngParams<Real>& p, cudaStream_t s) {
   constexpr int LA = pair_cls_la(X), LB = pair_cls_lb(X), LC = pair_cls_la(Y), LD = pair_cls_lb(Y);
   auto k = jeng_kernel<Real, LA, LB, LC, LD>;
   const size_t smem = jeng_smem_bytes<Real, LA, LB>(p.bra_ppmax);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // always the largest any handle needs, as launch_jk
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)jeng_smem_bytes<Real, LA, LB>(kMaxPrim * kMaxPrim));
   if (e != cudaSuccess || p.nitems == 0) return e;
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kJKThreads, smem);
