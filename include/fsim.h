@@ -136,7 +136,9 @@ int fsim_schwarz(fsim_basis* b, double* Q);
 typedef struct {
   double schwarz_tau;  /* skip unique quartets with Q_ab Q_cd < tau; 0 = no screening.  With tau > 0 a kept
                           quartet's contraction also leaves out primitive quartets whose own Schwarz
-                          bound is below min(2^-20 tau, 2^-53) (FSIM_MIXED: min(2^-13 tau, 2^-43)) */
+                          bound is below min(2^-61 Q_ab Q_cd, 2^-20 tau, 2^-53) (FSIM_MIXED:
+                          min(2^-32 Q_ab Q_cd, 2^-13 tau, 2^-43)): together at most 2^-53 (2^-24) of
+                          Q_ab Q_cd, so every integral keeps the accuracy of its precision */
   int precision;       /* FSIM_FP64, FSIM_MIXED or FSIM_DFLOAT */
   double boys_fp64_T;  /* mixed path: Boys to FP64-level accuracy (double-float arithmetic on the FP32
                           pipe, relative error <= 1e-13) for T >= this; 0 = never; values in (0, 30)

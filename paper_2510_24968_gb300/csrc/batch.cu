@@ -187,7 +187,7 @@ int build_tables(fsim_batch* bt, int prec) {
         if (cp.nitems == 0) continue;
         const Real* D = prec == 0 ? (const Real*)bt->h_ptrs[m].Din : (const Real*)bt->h_ptrs[m].D32;
         mols.push_back(JKMol<Real>{b->cls[X].view<Real>(), b->cls[Y].view<Real>(), cp.d_prefix, cp.d_count, b->nbf,
-                                   D, b->d_Jacc, b->d_Kacc, b->cls[X].d_Q, b->cls[Y].d_Q});
+                                   D, b->d_Jacc, b->d_Kacc});
         prefix.push_back(prefix.back() + cp.nitems);
         C.ids.push_back(m);
         C.bra_ppmax = std::max(C.bra_ppmax, b->cls[X].ppmax);

@@ -56,18 +56,23 @@ struct PairView {
   const typename Vec4<Real>::type* __restrict__ pq;  // (p, Px, Py, Pz) at [pp][pair]
   const float4* __restrict__ pe4;                    // FP32: E non-zeros by fours, [z / 4][pp][pair]
   const uint4* __restrict__ ub;                      // Schwarz bounds of the pair's primitive pairs (prim_mask)
+  const double* __restrict__ Q;                      // Schwarz bound of the pair
 };
 
 // Primitive quartets that cannot matter.  |(ab|cd)| of a primitive quartet is at
 // most q_ab q_cd, q_ab = sqrt(max_a |(ab_a|ab_a)|) of one primitive pair (Schwarz),
 // and the bounds of one contracted pair of distant centres span many orders of
 // magnitude.  A primitive quartet whose bound is below a threshold theta is left
-// out of the contraction: theta is a power of two at most 2^-20 of the screening
-// threshold and 2^-53 (FP64, double-float), or 2^-13 of it and 2^-43 (FP32), so
-// that all that is left out stays below the rounding of the integrals themselves
-// (prim_threshold; nothing is left out at screening threshold 0).  (H2O)_8 at
-// 1e-10 needs 60-70 % of its primitive quartets at the FP64 threshold (61.7 ->
-// 48.5 ms), the compact 7-atom cloud nearly all of them (55.4 ms both ways).
+// out of the contraction, where theta is a power of two that is at most
+//  * 2^-61 (FP64, double-float) or 2^-32 (FP32) of the contracted quartet's own
+//    Schwarz bound Q_ab Q_cd: all that is left out of a quartet, 256 primitive
+//    quartets at most, is within half a unit in the last place of that bound,
+//    however small the quartet is;
+//  * 2^-20 of the screening threshold and 2^-53 (FP32: 2^-13 of it and 2^-43), so
+//    that large FP32 integrals too keep the bits they have with nothing left out.
+// Nothing is left out at screening threshold 0.  Of the warps' steps (H2O)_8 at
+// 1e-10 keeps 89 % in FP64 and 70 % in FP32, the 12-atom cloud 95 and 84 %, the
+// compact 7-atom cloud all.
 //
 // Per pair, one byte per primitive pair: 0x80 | clamp(e + 96, 0, 127) with
 // q < 2^e; 127 means "no bound".
@@ -83,6 +88,21 @@ constexpr int kPrimKeepAll = -100000;  // log2 theta of an unscreened build
 template <typename Real>
 __host__ __device__ constexpr bool prim_skip(int L) {
   return std::is_same<Real, double>::value || (std::is_same<Real, float>::value ? L <= 4 : L <= 2);
+}
+
+// log2 theta relative to the quartet's own bound
+template <typename Real>
+constexpr int kPrimRel = std::is_same<Real, float>::value ? -32 : -61;
+// upper word of a pair's Schwarz bound: its exponent, biased, above bit 20
+__device__ __forceinline__ int bound_word(const double* Q, int i) {
+  return __ldg(reinterpret_cast<const int*>(Q) + 2 * (size_t)i + 1);
+}
+// log2 theta of a quartet from the build's (kPrimKeepAll stays) and its pairs' bound
+// words; a bound of zero or below the normal range keeps everything
+template <typename Real>
+__host__ __device__ __forceinline__ int prim_theta(int prim_lt, int wab, int wcd) {
+  const int own = (wab >> 20) + (wcd >> 20) - 2 * 1023 + kPrimRel<Real>;
+  return prim_lt < own ? prim_lt : own;
 }
 
 // byte of primitive pair b
@@ -117,8 +137,6 @@ struct JKMol {
   const Real* __restrict__ D;           // density, N x N, in the working precision
   double* J;                            // accumulators (FP64), N x N
   double* K;
-  const double* __restrict__ bq = nullptr;  // Schwarz bounds of the bra / ket class's pairs (same order);
-  const double* __restrict__ kq = nullptr;  // read only when JKParams::tau_mol is set
 };
 
 template <typename Real>
@@ -137,7 +155,7 @@ struct JKParams {
   int bra_ppmax;                        // largest bra primitive-pair count (shared-memory size)
   const Real* __restrict__ boys;
   float boys64_T;                       // FP32 path: Boys in FP64 at T >= this (infinity = never)
-  int prim_lt;                          // log2 of the primitive-quartet threshold (prim_mask)
+  int prim_lt;                          // log2 of the build's primitive-quartet threshold (prim_theta)
   // batched, optional: per molecule (indexed like active) a density-weighted
   // threshold; a quartet with Q_ab Q_cd below it is skipped (0: none skipped)
   const float* __restrict__ tau_mol = nullptr;
@@ -267,8 +285,8 @@ struct KetLoads {
 // a and ket components c = ch*CS + cs < NC, accumulated in this thread's
 // shared-memory slots so[(a * CS + cs) * kJKThreads] (so the registers hold
 // only R, the chunk's W and its E non-zeros).  Bra data: accessor bra(field, pp).
-// Primitive quartets below the threshold 2^prim_lt are skipped (prim_mask; bub:
-// the bra's bounds).
+// Primitive quartets below the quartet's threshold 2^prim_lt (prim_theta) are
+// skipped (prim_mask; bub: the bra's bounds).
 // The bstep threads of a quartet share its primitive quartets: with bstep <=
 // nppb each takes whole bra primitive pairs (b0, b0 + bstep, ...) and every ket
 // primitive pair; with more threads than bra primitive pairs the ket primitive
@@ -544,7 +562,7 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
       // density-weighted screening of an incremental build: every term this
       // quartet adds is bounded by Q_ab Q_cd max|dD|, compared here with tau / max|dD|
       const float te = __ldg(P.tau_mol + mol_id);
-      if (te > 0.0f && (float)(__ldg(M.bq + i) * __ldg(M.kq + j)) < te) valid = false;
+      if (te > 0.0f && (float)(__ldg(M.bra.Q + i) * __ldg(M.ket.Q + j)) < te) valid = false;
     }
     const int4 bi = i >= 0 ? M.bra.idx[i] : make_int4(0, 0, 0, 0);
 #pragma unroll
@@ -553,6 +571,9 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
       const int4 ki = valid ? M.ket.idx[j] : make_int4(0, 0, 0, 0);
       const int nppb = valid ? M.bra.npp[i] : 0;
       const int nppk = valid ? M.ket.npp[j] : 0;
+      int prim_lt = kPrimKeepAll;
+      if constexpr (prim_skip<Real>(L))
+        if (valid) prim_lt = prim_theta<Real>(P.prim_lt, bound_word(M.bra.Q, i), bound_word(M.ket.Q, j));
       const Real deg = Real((bi.z == bi.w ? 1 : 2) * (ki.z == ki.w ? 1 : 2) * ((P.same && i == j) ? 1 : 2));
       const size_t bstride = (size_t)M.bra.ppmax * M.bra.n;
       const Real* bpd = M.bra.pd + (i >= 0 ? i : 0);
@@ -570,7 +591,7 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
 #pragma unroll 1
       for (int ch = cg; ch < KetChunks<KC, CS>::NCH; ch += ncg) {
         if (valid)
-          quartet_chunk<Real, LA, LB, LC, LD, CS>(so, bra, nppb, bs, ps, M.ket, j, nppk, M.bra.ub + i, P.prim_lt,
+          quartet_chunk<Real, LA, LB, LC, LD, CS>(so, bra, nppb, bs, ps, M.ket, j, nppk, M.bra.ub + i, prim_lt,
                                                   sBoys, BK, P.boys64_T, ch);
         if (ps > 1) {
           // the ps threads of a quartet hold partial blocks over their bra

@@ -76,15 +76,15 @@ struct DevClass {
 
 template <>
 inline PairView<double> DevClass::view<double>() const {
-  return PairView<double>{n, ppmax, idx, npp, pd64, pq64, nullptr, ub};
+  return PairView<double>{n, ppmax, idx, npp, pd64, pq64, nullptr, ub, d_Q};
 }
 template <>
 inline PairView<float> DevClass::view<float>() const {
-  return PairView<float>{n, ppmax, idx, npp, pd32, pq32, pe32, ub};
+  return PairView<float>{n, ppmax, idx, npp, pd32, pq32, pe32, ub, d_Q};
 }
 template <>
 inline PairView<dfloat> DevClass::view<dfloat>() const {
-  return PairView<dfloat>{n, ppmax, idx, npp, pdx, pqx, nullptr, ub};
+  return PairView<dfloat>{n, ppmax, idx, npp, pdx, pqx, nullptr, ub, d_Q};
 }
 
 // Ket components per register chunk.  The per-thread registers of the unrolled
@@ -186,7 +186,7 @@ struct ClassPairPlan {
   int coop = 0;             // 1: table-driven kernel, a warp (FP32) or a CTA (FP64) per quartet
   int fp64 = 0;             // FSIM_DFLOAT plans: 1 = this class pair runs the FP64 kernel
   int tq = kJKThreads;      // kets per work item
-  int prim_lt = kPrimKeepAll;  // log2 of the primitive-quartet threshold
+  int prim_lt = kPrimKeepAll;  // log2 of the build's primitive-quartet threshold (prim_theta)
   int* d_prefix = nullptr;  // [nbra + 1]
   int* d_count = nullptr;   // [nbra]
 };
@@ -295,7 +295,7 @@ struct fsim_basis {
 };
 
 namespace fsim {
-// log2 of the primitive-quartet threshold of a build screened at tau (prim_mask)
+// log2 of the primitive-quartet threshold of a build screened at tau (prim_theta)
 int prim_threshold(double tau, bool fp32);
 // the Boys table the quartet kernels of a precision stage (stage_boys)
 template <typename Real>

@@ -134,6 +134,9 @@ __global__ void __launch_bounds__(kGenThreads, 4) gen_kernel(GenParams<Real> P) 
     const int nppb = P.bra.npp[i], nppk = P.ket.npp[j];
     const int b_lo = share * nppb / P.nsplit, b_hi = (share + 1) * nppb / P.nsplit;  // this CTA's bra primitive pairs
     if (b_lo == b_hi) continue;
+    const int prim_lt = P.prim_lt == kPrimKeepAll  // (the bounds themselves are made so, before Q exists)
+                            ? kPrimKeepAll
+                            : prim_theta<Real>(P.prim_lt, bound_word(P.bra.Q, i), bound_word(P.ket.Q, j));
     const Real* bp = P.bra.pd + i;
     const Real* kp = P.ket.pd + j;
     const int4 bi = P.bra.idx[i], ki = P.ket.idx[j];
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(kGenThreads, 4) gen_kernel(GenParams<Real> P) 
           const int b = tid / nk, k = k0 + tid % nk;
           bool keep = false;
           if (tid < nb * nk)
-            keep = P.prim_lt == kPrimKeepAll || prim_byte(P.ket.ub + j, k) >= prim_least(P.prim_lt, prim_byte(P.bra.ub + i, b0 + b));
+            keep = prim_lt == kPrimKeepAll || prim_byte(P.ket.ub + j, k) >= prim_least(prim_lt, prim_byte(P.bra.ub + i, b0 + b));
           const unsigned bal = __ballot_sync(0xffffffffu, keep);
           if ((tid & 31) == 0) sCnt[tid >> 5] = __popc(bal);
           __syncthreads();  // (also: the previous step's columns have been read)

@@ -68,7 +68,7 @@ struct GenParams {
   double* K;
   const Real* __restrict__ boys;     // full table, rows of kBoysCols
   float boys64_T;
-  int prim_lt;                       // log2 of the primitive-quartet threshold (prim_mask)
+  int prim_lt;                       // log2 of the build's primitive-quartet threshold (prim_theta)
   GenLayout lay;                     // filled by launch_gen
 };
 

@@ -34,7 +34,7 @@ struct JEngParams {
   int bra_ppmax;
   const Real* __restrict__ boys;
   float boys64_T;
-  int prim_lt;                        // log2 of the primitive-quartet threshold (prim_mask)
+  int prim_lt;                        // log2 of the build's primitive-quartet threshold (prim_theta)
 };
 
 // How the FP32 kernels load a ket's data (as KetLoads of eri_core.cuh, for the same
@@ -133,10 +133,13 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
     const int j = tile * tq + q;
     if (q < tq && j < __ldg(P.ket_count + i)) {
       const int nppk = P.ket.npp[j];
+      int prim_lt = kPrimKeepAll;
+      if constexpr (prim_skip<Real>(L))
+        prim_lt = prim_theta<Real>(P.prim_lt, bound_word(P.bra.Q, i), bound_word(P.ket.Q, j));
       for (int b = bs; b < nppb; b += ps) {
         unsigned todo = (1u << nppk) - 1u;
         if constexpr (prim_skip<Real>(L)) {
-          todo = prim_mask(__ldg(P.ket.ub + j), prim_least(P.prim_lt, prim_byte(P.bra.ub + i, b)), nppk);
+          todo = prim_mask(__ldg(P.ket.ub + j), prim_least(prim_lt, prim_byte(P.bra.ub + i, b)), nppk);
           if (todo == 0) continue;
         }
         const Real* sb = sbra + b * NFB;
