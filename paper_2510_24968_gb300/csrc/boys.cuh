@@ -201,41 +201,53 @@ __device__ __forceinline__ double rsqrt_fp64(double x) {
 //    leaves i in the low word: no conversions; range check on the high word.
 //  * e^{-T} = e^{-T_i} e^{x}, |x| <= 1/32, Taylor to x^7 (next term < 2^-55),
 //    in place of the library exponential.
-//  * T >= 36: F_0 from rsqrt_fp64.  e^{-T} <= 2.4e-16; taken from FP32 (2e-6 of
-//    it, mostly from rounding T) it leaves 1e-16 of F_5 at T = 36 and less of
-//    lower orders; from order 6 on it is the FP64 exponential.
+//  * T >= 36: F_0 from rsqrt_fp64 and upward recursion.  e^{-T} (at most 2.4e-16) up
+//    to T = 72 as the square of e^{-T/2}; beyond, it is below 2^-59 of the term it
+//    would be subtracted from in every order up to 12.  The exponential comes before
+//    the branch, so that a warp on both sides evaluates it once.
 // One (ps|ss) primitive quartet went from 67 to about 46 FP64 instructions with
 // this and rsqrt_fp64 (ncu: pipe share times duration).
 template <int K>
 constexpr double inv_fact_c = inv_fact(K);  // a constant in device code too, never a call
 constexpr double kBoysRound = 422212465065984.0;  // 3 2^47
+// Upper words of -72 and -144 (T = 36 and 72): for u <= 0 the larger -u, the larger
+// the word as an integer.
+constexpr int kBoysWord36 = (int)0xC0520000, kBoysWord72 = (int)0xC0620000;
+// T < 36: e^{-T}; 36 <= T < 72: e^{-T/2} (T >= 72: 0).  x = T_i - T and the row of T_i of
+// the T or T/2 taken come back too.
+__device__ __forceinline__ double boys_exp(double u, const double* __restrict__ tabL, int stride, int ecol, double& x,
+                                           const double*& row) {
+  const int w = __double2hiint(u);
+  if (w >= kBoysWord72) return 0.0;
+  const double v = w >= kBoysWord36 ? __hiloint2double(w - 0x00100000, __double2loint(u)) : u;
+  const double t = fma(v, -0.5, kBoysRound);
+  x = fma(v, 0.5, t - kBoysRound);
+  row = tabL + __double2loint(t) * stride;
+  constexpr int kExpTerms = 7;
+  double ex = inv_fact_c<kExpTerms>;
+  static_for<kExpTerms>([&](auto I) { ex = fma(ex, x, inv_fact_c<kExpTerms - 1 - decltype(I)::value>); });
+  return row[ecol] * ex;
+}
 template <int L, bool SCALED>
 __device__ __forceinline__ void boys_fp64_u(double u, double (&F)[L + 1], const double* __restrict__ tabL, int stride,
                                             int ecol) {
-  if (__double2hiint(u) < (int)0xC0520000) {  // as integers, for u <= 0: -u < 72
-    const double t = fma(u, -0.5, kBoysRound);
-    const double Ti = t - kBoysRound;
-    const double x = fma(u, 0.5, Ti);  // -(T - T_i)
-    const double* row = tabL + __double2loint(t) * stride;
+  double x = 0.0;
+  const double* row = tabL;
+  const double e = boys_exp(u, tabL, stride, ecol, x, row);
+  if (__double2hiint(u) < kBoysWord36) {
     double acc = row[kBoysK64 - 1];
 #pragma unroll
     for (int k = kBoysK64 - 1; k >= 1; --k) acc = fma(acc, SCALED ? x : x * inv_int(k), row[k - 1]);
     F[L] = acc;
-    if constexpr (L > 0) {
-      constexpr int kExpTerms = 7;
-      double ex = inv_fact_c<kExpTerms>;
-      static_for<kExpTerms>([&](auto I) { ex = fma(ex, x, inv_fact_c<kExpTerms - 1 - decltype(I)::value>); });
-      const double e = row[ecol] * ex;
 #pragma unroll
-      for (int n = L - 1; n >= 0; --n) F[n] = n > 0 ? fma(-u, F[n + 1], e) * inv_odd(n) : fma(-u, F[1], e);
-    }
+    for (int n = L - 1; n >= 0; --n) F[n] = n > 0 ? fma(-u, F[n + 1], e) * inv_odd(n) : fma(-u, F[1], e);
   } else {
     const double rs = rsqrt_fp64(-0.5 * u);
     F[0] = 0.5 * kSqrtPi * rs;
     if constexpr (L > 0) {
-      const double h = 0.5 * rs * rs, e = L <= 5 ? (double)expf(0.5f * (float)u) : exp(0.5 * u);
+      const double h = 0.5 * rs * rs, eT = e * e;
 #pragma unroll
-      for (int n = 1; n <= L; ++n) F[n] = ((2 * n - 1) * F[n - 1] - e) * h;
+      for (int n = 1; n <= L; ++n) F[n] = ((2 * n - 1) * F[n - 1] - eT) * h;
     }
   }
 }
