@@ -126,6 +126,15 @@ __host__ __device__ __forceinline__ unsigned prim_mask(uint4 v, int least, int n
   return m & ((1u << npp) - 1u);
 }
 
+// The work items of a persistent CTA: first, first + step, ... below n.  Unsigned: a
+// launch may have nearly 2^31 items, and the step past the last must not wrap.
+struct ItemLoop {
+  unsigned i, step, n;
+  __host__ __device__ ItemLoop(unsigned first, unsigned step_, int n_) : i(first), step(step_), n((unsigned)n_) {}
+  __host__ __device__ bool more() const { return i < n; }
+  __host__ __device__ void next() { i += step; }
+};
+
 // Everything a work item needs about its molecule.
 template <typename Real>
 struct JKMol {
@@ -519,7 +528,8 @@ __global__ void __launch_bounds__(kJKThreads) jk_kernel(JKParams<Real> P) {
   Real* so = sOut + threadIdx.x;
   Real* jb = sJb + threadIdx.x;  // this thread's part of J_acc for its bra block, jb[a * kJKThreads]
 
-  for (int item = blockIdx.x; item < P.nitems; item += gridDim.x) {
+  for (ItemLoop at(blockIdx.x, gridDim.x, P.nitems); at.more(); at.next()) {
+    const int item = (int)at.i;
     int litem = item;
     int mol_id = 0;
     const JKMol<Real>* Mp = &P.one;

@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(kGenThreads, 4) gen_kernel(GenParams<Real> P) 
   if (tid < 16) sCoef[tid] = Real(tid);
   __syncthreads();
   const size_t bstride = (size_t)P.bra.ppmax * P.bra.n, kstride = (size_t)P.ket.ppmax * P.ket.n;
-  for (int it = blockIdx.x; it < P.nitems * P.nsplit; it += gridDim.x) {
-    const int q = it / P.nsplit, share = it - q * P.nsplit;
+  for (ItemLoop at(blockIdx.x, gridDim.x, P.nitems * P.nsplit); at.more(); at.next()) {
+    const int q = (int)at.i / P.nsplit, share = (int)at.i - q * P.nsplit;
     int i, j;
     if (P.list_mode) {
       const int2 it = P.items[q];

@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(kJKThreads) jeng_kernel(JEngParams<Real> P) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Real* jslot = sJ + threadIdx.x;
   const size_t kstride = (size_t)P.ket.ppmax * P.ket.n;
-  for (int item = blockIdx.x; item < P.nitems; item += gridDim.x) {
+  for (ItemLoop at(blockIdx.x, gridDim.x, P.nitems); at.more(); at.next()) {
+    const int item = (int)at.i;
     const int i = find_bra(P.prefix, P.bra.n, item);
     const int tile = item - __ldg(P.prefix + i);
     const int nppb = P.bra.npp[i];
