@@ -226,8 +226,8 @@ int fsim_j_build(fsim_basis* b, const double* D, double* J, const fsim_fock_opts
  * FP64 cooperative kernel where the untuned plan has it.  choice (36 entries,
  * optional): 10 * psplit + csplit for the unrolled kernel (+ 1000 when a
  * double-float build runs the class pair with the FP64 kernel), -1 for the
- * cooperative kernel (FSIM_DFLOAT: 0, as planned), 0 for class pairs without
- * work; best_ms (36, optional): its median time.  Index X*6+Y as in
+ * cooperative kernel (FSIM_DFLOAT: 1000, the FP64 one), 0 for class pairs
+ * without work; best_ms (36, optional): its median time.  Index X*6+Y as in
  * fsim_last_class_times.
  */
 int fsim_autotune(fsim_basis* b, const fsim_fock_opts* opts, int* choice, float* best_ms);
@@ -239,8 +239,8 @@ int fsim_autotune(fsim_basis* b, const fsim_fock_opts* opts, int* choice, float*
  * it is.  Errors (FSIM_EINVAL, plan unchanged for that and later class pairs):
  * psplit not 1/3/9 or above the bra class's primitive pairs (27: bra class
  * below 9 or ket class below 3 primitive pairs), csplit not 1/2/4 or above its
- * ket chunks, the cooperative kernel with FSIM_DFLOAT, +1000 outside
- * FSIM_DFLOAT, or the double-float kernel for (dd|dp) and (dd|dd).
+ * ket chunks, -1 with FSIM_DFLOAT (1000 is its cooperative kernel), 1000 and
+ * above outside FSIM_DFLOAT, or the double-float kernel for (dd|dp) and (dd|dd).
  */
 int fsim_set_launch(fsim_basis* b, const fsim_fock_opts* opts, const int* choice);
 

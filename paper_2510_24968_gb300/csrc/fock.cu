@@ -867,6 +867,11 @@ int fock_build_into(fsim_basis* b, const double* dD, double* dJ, double* dK, con
 
 namespace fsim {
 
+// fsim_autotune's code of the FP64 cooperative kernel in double-float plans (+ 1000 as
+// for every FP64 shape there, no threads per quartet; positive, as all codes of a
+// double-float plan)
+constexpr int kCoop64Choice = 1000;
+
 template <typename Real>
 static int autotune_impl(fsim_basis* b, FockPlan* plan, const Real* Dr, float b64, cudaStream_t s, int* choice,
                          float* best_ms, const double* D64 = nullptr) {
@@ -897,8 +902,8 @@ static int autotune_impl(fsim_basis* b, FockPlan* plan, const Real* Dr, float b6
           for (int cs : {1, 2, 4})
             if (psplit_legal(b, X, Y, ps) && cs <= nch && (ps < 27 || cp.nquartets * 9 < fill))
               cands.push_back({ps, 0, cs, f64});
-      // the cooperative kernel; a double-float build has it where it is the
-      // class pair's default (reported as 0, fsim_set_launch's "as planned")
+      // the cooperative kernel; a double-float build has the FP64 one where it is
+      // the class pair's default
       if (!kDf) cands.push_back({1, 1, 1, 0});
       else if (plan_gen64(FSIM_DFLOAT, X, Y, cp.nquartets)) cands.push_back({1, 1, 1, 1});
       float best = 1e30f;
@@ -934,7 +939,7 @@ static int autotune_impl(fsim_basis* b, FockPlan* plan, const Real* Dr, float b6
       if (rc != FSIM_OK) break;
       rc = set_class_plan(b, X, Y, count, win.psplit, win.coop, cp, win.csplit, jk_flat<Real>());
       cp.fp64 = win.fp64;
-      if (choice) choice[ci] = win.coop ? (kDf ? 0 : -1) : 10 * win.psplit + win.csplit + 1000 * win.fp64;
+      if (choice) choice[ci] = win.coop ? (kDf ? kCoop64Choice : -1) : 10 * win.psplit + win.csplit + 1000 * win.fp64;
       if (best_ms) best_ms[ci] = best;
     }
   cudaEventDestroy(e0);
@@ -964,11 +969,10 @@ extern "C" int fsim_set_launch(fsim_basis* b, const fsim_fock_opts* opts, const 
       const int c = choice[X * kNumPairCls + Y];
       ClassPairPlan& cp = plan->cp[X][Y];
       if (c == 0 || cp.nquartets == 0) continue;
-      const int coop = c == -1 ? 1 : 0;
+      const int coop = c == (df ? kCoop64Choice : -1) ? 1 : 0;
       const int f64 = c >= 1000 ? 1 : 0, ps = coop ? 1 : (c % 1000) / 10, cs = coop ? 1 : c % 10;
-      const bool ok = c >= -1 && c < 2000 && (coop ? !df : (psplit_legal(b, X, Y, ps) &&
-                                                          (cs == 1 || cs == 2 || cs == 4) &&
-                                                          cs <= jk_chunks_precision(o.precision, X, Y))) &&
+      const bool ok = (coop || (c > 0 && c < 2000 && psplit_legal(b, X, Y, ps) && (cs == 1 || cs == 2 || cs == 4) &&
+                                cs <= jk_chunks_precision(o.precision, X, Y))) &&
                       (!f64 || df) && (!df || f64 || dfloat_kernel(X, Y));
       if (!ok) {
         set_error("fsim_set_launch: choice %d not valid for class pair (%d|%d) in precision %d", c, X, Y, o.precision);
