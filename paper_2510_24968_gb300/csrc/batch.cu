@@ -182,13 +182,17 @@ int build_tables(fsim_batch* bt, int prec) {
       for (int m = 0; m < bt->nmol; ++m) {
         fsim_basis* b = bt->b[m];
         FockPlan* plan = nullptr;
-        FSIM_TRY(get_plan(b, bt->tau, 0, 1, prec == 0 ? FSIM_FP64 : FSIM_MIXED, &plan, C.psplit));
+        FSIM_TRY(get_plan(b, bt->tau, 0, 1, prec == 0 ? FSIM_FP64 : FSIM_MIXED, &plan, 1));
         const ClassPairPlan& cp = plan->cp[X][Y];
         if (cp.nitems == 0) continue;
+        // the FP64 kernel's lists are flat, the same for every split; only the
+        // quartets a tile takes differ
+        static_assert(jk_flat<double>(), "nine threads a quartet on the plan's own lists");
+        const long long tq = kJKThreads / C.psplit;
         const Real* D = prec == 0 ? (const Real*)bt->h_ptrs[m].Din : (const Real*)bt->h_ptrs[m].D32;
         mols.push_back(JKMol<Real>{b->cls[X].view<Real>(), b->cls[Y].view<Real>(), cp.d_prefix, cp.d_count, b->nbf,
                                    D, b->d_Jacc, b->d_Kacc});
-        prefix.push_back(prefix.back() + cp.nitems);
+        prefix.push_back(prefix.back() + (C.psplit > 1 ? (int)((cp.nquartets + tq - 1) / tq) : cp.nitems));
         C.ids.push_back(m);
         C.bra_ppmax = std::max(C.bra_ppmax, b->cls[X].ppmax);
       }
