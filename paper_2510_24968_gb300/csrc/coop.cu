@@ -1,4 +1,4 @@
-// Warp-cooperative quartet kernel instantiations (FP64 and FP32).
+// Warp-cooperative quartet kernel instantiations (FP64: quartet lists; FP32: J/K).
 #include "coop.cuh"
 namespace fsim {
 template cudaError_t launch_coop<double>(const CoopParams<double>&, int, cudaStream_t);

@@ -9,8 +9,9 @@
 //   * W[h][c] (ket transform) and out[a][c] (bra transform) distributed over
 //     the lanes, W passed through shared memory between the two transforms.
 // Loops run over runtime index tables, so one compiled kernel serves every
-// class pair.  Used for explicit quartet lists (Schwarz diagonal, debug dumps)
-// and as one of the autotuner's launch shapes for the J/K build.
+// class pair.  In FP64 it evaluates explicit quartet lists (Schwarz diagonal, debug
+// dumps); in FP32 it is one of the autotuner's launch shapes of the J/K build (the
+// FP64 one is the CTA-per-quartet kernel of generic.cuh).
 #pragma once
 #include "eri_core.cuh"
 
@@ -58,14 +59,13 @@ struct CoopParams {
   PairView<Real> bra, ket;
   ClsDesc bd, kd;
   int same;
-  // JK mode (items from tile prefix) or list mode (explicit items)
-  int list_mode;
+  // FP32, J/K: items from the tile prefix; FP64: explicit items
   const int* __restrict__ tile_prefix;
   const int* __restrict__ ket_count;
   int tq;  // kets per work item
   const int2* __restrict__ items;
   int nitems;
-  double* out;  // list mode: block per item
+  double* out;  // FP64: block per item
   int N;
   const Real* __restrict__ D;
   double* J;
@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(kCoopWarps * 32) coop_kernel(CoopParams<Real> 
   __syncthreads();
   const ClsDesc& bd = sbd;
   const ClsDesc& kd = skd;
+  constexpr bool kList = std::is_same<Real, double>::value;
   const int L = bd.L + kd.L;
   const int S = L + 1;
   Real* R = sRall + (size_t)warp * (kCoopCube + kCoopWsize);
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(kCoopWarps * 32) coop_kernel(CoopParams<Real> 
 
   // quartet assignment
   int i = 0, j0 = 0, jn = 0;
-  if (P.list_mode) {
+  if constexpr (kList) {
     const int t = blockIdx.x * kCoopWarps + warp;
     if (t < P.nitems) {
       i = P.items[t].x;
@@ -151,8 +152,8 @@ __global__ void __launch_bounds__(kCoopWarps * 32) coop_kernel(CoopParams<Real> 
   }
   const int4 bi = P.bra.idx[i];
   const int nppb = P.bra.npp[i];
-  for (int qq = (P.list_mode ? 0 : warp); qq < jn; qq += (P.list_mode ? 1 : kCoopWarps)) {
-    const int j = P.list_mode ? j0 : j0 + qq;
+  for (int qq = kList ? 0 : warp; qq < jn; qq += kList ? 1 : kCoopWarps) {
+    const int j = kList ? j0 : j0 + qq;
     const int4 ki = P.ket.idx[j];
     const int nppk = P.ket.npp[j];
     Real outv[kCoopMaxOut];
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(kCoopWarps * 32) coop_kernel(CoopParams<Real> 
       __syncwarp();
     }
     // emit
-    if (P.list_mode) {
+    if constexpr (kList) {
       double* o = P.out + (size_t)(blockIdx.x * kCoopWarps + warp) * NO;
 #pragma unroll
       for (int m = 0; m < kCoopMaxOut; ++m) {

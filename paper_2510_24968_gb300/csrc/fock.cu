@@ -99,7 +99,6 @@ int run_list(fsim_basis* b, int X, int Y, const std::vector<int2>& items, double
     p.ket = b->cls[Y].view<double>();
     make_cls_desc(X, p.bd);
     make_cls_desc(Y, p.kd);
-    p.list_mode = 1;
     p.items = d_items;
     p.nitems = (int)items.size();
     p.out = d_out;
@@ -388,7 +387,6 @@ static cudaError_t launch_cp(fsim_basis* b, int X, int Y, const ClassPairPlan& c
       make_cls_desc(X, p.bd);
       make_cls_desc(Y, p.kd);
       p.same = X == Y ? 1 : 0;
-      p.list_mode = 0;
       p.tile_prefix = cp.d_prefix;
       p.ket_count = cp.d_count;
       p.tq = cp.tq;
