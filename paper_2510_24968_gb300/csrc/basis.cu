@@ -73,7 +73,6 @@ static cudaError_t launch_pair_data(int cls, int n, int ppmax, const int4* idx, 
   return cudaGetLastError();
 }
 
-// (Re)build the device data of pair class `cls` in the given pair order.
 // E non-zeros of the FP32 pair data by fours: the quartet kernels load a ket's in
 // 16-byte words.  One thread per (group of four, primitive pair, pair).
 __global__ void pair_quads_kernel(int nnz, size_t fs, const float* __restrict__ pd, float4* __restrict__ pe) {
@@ -85,6 +84,7 @@ __global__ void pair_quads_kernel(int nnz, size_t fs, const float* __restrict__ 
   pe[x] = make_float4(e[0], e[1], e[2], e[3]);
 }
 
+// (Re)build the device data of pair class `cls` in the given pair order.
 int build_pair_data(fsim_basis* b, int cls, const std::vector<int4>& order) {
   DevClass& C = b->cls[cls];
   dev_free(C.idx); dev_free(C.npp); dev_free(C.pd64); dev_free(C.pd32); dev_free(C.pq64); dev_free(C.pq32);
@@ -178,9 +178,8 @@ __global__ void split4_kernel(const double4_32a* __restrict__ in, dfloat4* __res
   }
 }
 
-// The double-float table keeps e^{-T_i} in its last column (an order no class
-// reaches), read by the double-float Boys function.
-// Per-order tables of the quartet kernels from the full FP64 table (stage_boys).
+// Per-order tables of the quartet kernels from the full FP64 table (stage_boys): FP64
+// with F_{L+k} / k!, double-float with F_{L+k}; the last slot is e^{-T_i} in both.
 template <typename Real>
 __global__ void boys_orders_kernel(const double* __restrict__ full, Real* __restrict__ out) {
   constexpr int NC = Boys<Real>::NCOL;

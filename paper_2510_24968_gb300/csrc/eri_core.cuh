@@ -80,11 +80,15 @@ constexpr int kPrimBias = 96, kPrimNoBound = 127;
 constexpr int kPrimKeepAll = -100000;  // log2 theta of an unscreened build
 
 // Kernels of order L that skip: FP64 (bound by its arithmetic) all of them; FP32
-// and double-float those whose unrolled bodies are short.  The others are bound
+// and double-float those whose unrolled bodies are short (the CTA-per-quartet kernel
+// of generic.cuh, which has none, skips at every order).  The others are bound
 // by instruction supply, which their warps share while they run in step, and
 // skipping puts them out of step (30-atom cloud, FP32: (dp|ps) 46 -> 38 ms, but
 // (dd|dp) 60 -> 77; 12-atom cloud: (dp|pp) 2.14 -> 2.26; (H2O)_8, double-float:
-// (ps|ss) 1.47 -> 1.08 ms, but (dp|ps) 1.9 -> 4.3).
+// (ps|ss) 1.47 -> 1.08 ms, but (dp|ps) 1.9 -> 4.3; all at the second threshold above
+// alone, which leaves out more).  Whole builds with and without: (H2O)_8 FP64 57.7 ms
+// against 61.7 with nothing left out, mixed 3.23 against 3.40, J alone 2.05 against
+// 2.53; 30-atom cloud, mixed, 566 against 602; double-float even.
 template <typename Real>
 __host__ __device__ constexpr bool prim_skip(int L) {
   return std::is_same<Real, double>::value || (std::is_same<Real, float>::value ? L <= 4 : L <= 2);

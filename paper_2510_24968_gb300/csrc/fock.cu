@@ -200,10 +200,11 @@ int prim_threshold(double tau, bool fp32) {
 }
 
 // Whether a build evaluates a class pair in FP64 with a CTA per quartet: the
-// heavy class pairs, and those with at most two waves of its CTAs, where the
-// unrolled kernel's threads, nine to a quartet, leave the FP64 pipes idle (six
-// (pp|pp) quartets: 35 against 201 us; 560 (pp|ps): 49 against 78; 1050
-// (pp|ss): 53 against 43).
+// heavy class pairs, and those with at most six of its CTAs to an SM, where the
+// unrolled kernel's threads, nine or 27 to a quartet, leave the FP64 pipes idle (six
+// (pp|pp) quartets: 26 against 111 us in its best shape; 231: 49 against 115; 560
+// (pp|ps): 35 against 47; but 1050 (pp|ss): 45 against 37; 1596 (ps|ps): 57 against
+// 51; 2646 (pp|ps): even).
 static bool plan_gen64(int precision, int X, int Y, long long nquartets) {
   const bool in64 = precision == FSIM_FP64 || (precision == FSIM_DFLOAT && !dfloat_default(X, Y));
   return in64 && (gen64_default(X, Y) || nquartets <= 6 * device_sm_count());

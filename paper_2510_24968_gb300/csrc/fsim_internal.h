@@ -154,7 +154,7 @@ __host__ __device__ constexpr int chunk_size(int X, int Y) {
 __host__ __device__ constexpr bool dfloat_kernel(int X, int Y) { return !(X == 5 && Y >= 4); }
 // Default kernel of a class pair in an FSIM_DFLOAT build (the autotuner times
 // both): double-float up to total angular momentum 4, where the Boys function
-// and the prologue weigh most (measured on (H2O)_8: 3-8x faster than FP64);
+// and the prologue weigh most (measured on (H2O)_8: 1.7-4.7x faster than FP64, (pp|pp) even);
 // FP64 from 5, where R and the chunk's W outgrow 255 registers at two per value
 // and live in L1-backed local memory, which the double-float kernel, at 15 FP32
 // instructions per multiply-add, cannot feed fast enough: the two run even.
@@ -164,7 +164,12 @@ __host__ __device__ constexpr bool dfloat_default(int X, int Y) {
 // Class pairs whose FP64 evaluation takes the CTA-per-quartet kernel
 // (generic.cuh) instead of the unrolled one: where the ket transform, H(bra) x
 // non-zeros(ket) multiply-adds per primitive quartet, outweighs what the former
-// spends per primitive quartet at 27 of 32 lanes.
+// spends per primitive quartet at 27 of 32 lanes.  12-atom cloud, against the unrolled
+// kernel's best shape: (dp|pp), product 660, 49.8 against 56.0 ms, (dd|pp) 18.3 against
+// 25.2, (dd|ds) 10.5 against 13.5; below the line (dp|ds), 420, 33.0 against 28.2,
+// (pp|pp), 330, 20.4 against 17.4, (dd|ps), 210, 14.9 against 12.3.  Smaller launches
+// are closer there: 7-atom cloud (pp|pp) 2.94 against 2.92, (dd|ps) 2.05 against 1.79,
+// (H2O)_8 0.77 against 0.83 and 2.45 against 2.64.
 __host__ __device__ constexpr bool gen64_default(int X, int Y) {
   return nherm(pair_cls_la(X) + pair_cls_lb(X)) * pair_cls_nnz(Y) >= 600;
 }

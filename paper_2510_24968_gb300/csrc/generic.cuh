@@ -17,8 +17,8 @@
 //   3. out[a][c] += sum_b sum_{h in nz(a)} E^{ab,b}_{a,h} W[b][c][h];
 // and per quartet the digestion: each thread sums one element of the J/K
 // blocks over the quartet block and adds it with one FP64 atomic.
-// Five barriers per group, none per primitive quartet or recursion level.  An
-// FP64 launch with fewer quartets than resident CTAs shares each quartet's bra
+// Four barriers per group and two per quartet, none per primitive quartet or
+// recursion level.  An FP64 launch with fewer quartets than resident CTAs shares each quartet's bra
 // primitive pairs out over several CTAs, which digest their partial blocks
 // (six (dd|dd) quartets: 0.77 ms with one CTA each).
 //
@@ -30,8 +30,9 @@
 // kernel of eri_core.cuh repeats R for every ket chunk and, at one warp per
 // scheduler, waits on its local-memory arrays: it used 50-65 % of the FP64 pipe.
 // 64 registers a thread let a fourth CTA onto the SM where its shared memory fits,
-// to fill the others' barriers ((H2O)_8 FP64 48.1 -> 47.3 ms, f shells 18.0 -> 16.8);
-// groups cut down so that four always fit gain nothing more (47.7, 17.0).
+// to fill the others' barriers ((H2O)_8 FP64 build -1.7 %, (H2O)_3 with f shells -7 %);
+// groups cut down so that four always fit gain nothing more (+0.8, +1 %).  On a
+// 7-atom cloud it uses 78-91 % of the FP64 pipe.
 #pragma once
 #include "eri_core.cuh"
 
