@@ -347,9 +347,18 @@ int backward32(fsim_mlp* n, const float* x, const float* t, const float* mask, i
 }
 
 // ---- BF16 path
-constexpr int kMaxSplits = 32;  // of the batch in the weight gradients
 inline int row_tiles(int b) { return (b + kTcM - 1) / kTcM; }
-inline int split_rows(int b) { return (row_tiles(b) + kMaxSplits - 1) / kMaxSplits * kTcM; }
+// Splits of the batch in the weight gradients: enough for four CTAs an SM, 32 at most
+// (width 256: 10 tiles, 32 splits).  Each keeps a copy of the gradient, so a wide
+// network, whose tiles fill the device by themselves, takes few.
+int max_splits(const fsim_mlp* n) {
+  const long long ti = row_tiles(n->nin), tw = row_tiles(n->width), to = row_tiles(n->nout);
+  return (int)std::max(1LL, std::min(32LL, 4LL * device_sm_count() / (ti * tw + tw * tw + tw * to)));
+}
+int split_rows(const fsim_mlp* n, int b) {
+  const int most = max_splits(n);
+  return (row_tiles(b) + most - 1) / most * kTcM;
+}
 
 template <typename T>
 int regrow(T** p, size_t n) {
@@ -378,7 +387,7 @@ int ensure_backward(fsim_mlp* n, int b) {
   FSIM_TRY(regrow(&n->dyb, bs * tc_ld(n->nout)));
   FSIM_TRY(regrow(&n->d1b, bs * lw));
   FSIM_TRY(regrow(&n->d2b, bs * lw));
-  FSIM_TRY(regrow(&n->part, (size_t)std::min(row_tiles(b), kMaxSplits) * n->np));
+  FSIM_TRY(regrow(&n->part, (size_t)std::min(row_tiles(b), max_splits(n)) * n->np));
   FSIM_TRY(regrow(&n->partb, row_tiles(b) * (nb + (tc_ld(n->nout) + kTcN - 1) / kTcN)));
   n->maxbg = b;
   return FSIM_OK;
@@ -439,7 +448,7 @@ int grad16(fsim_mlp* n, const float* x, const float* t, const float* mask, int b
   g.part = n->part;
   g.np = n->np;
   g.batch = b;
-  g.rows = split_rows(b);
+  g.rows = split_rows(n, b);
   const int nsplit = (b + g.rows - 1) / g.rows;
   constexpr int smem = tc_smem(kTcWStages);
   FSIM_CK(cudaFuncSetAttribute(tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
